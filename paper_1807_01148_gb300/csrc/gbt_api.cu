@@ -18,7 +18,7 @@ void launch_step(const Dev& d, int grid, bool has_stop, cudaStream_t s);
 void launch_occupancy(const Dev& d, int grid, cudaStream_t s);
 void launch_count(const Dev& d, int grid, cudaStream_t s);
 int scan_blocks(int n_lanes);
-void launch_state_out(const Dev& d, int grid, cudaStream_t s, uint8_t* status, int32_t* link, int32_t* lane,
+void launch_state_out(const Dev& d, int grid, cudaStream_t s, bool seg, uint8_t* status, int32_t* link, int32_t* lane,
                       int32_t* cursor, float* x, float* v, int32_t* ins, int32_t* arr, int8_t* dec);
 void launch_state_in(const Dev& d, int grid, cudaStream_t s, const uint8_t* status, const int32_t* link,
                      const int32_t* lane, const int32_t* cursor, const float* x, const float* v);
@@ -51,6 +51,19 @@ void launch_fw_final_time(const double* t0, const double* x, const double* cap, 
                           int n, cudaStream_t s);
 void launch_compact_routes(const int32_t* roff, const int32_t* rlen, const int32_t* src, const int32_t* new_off,
                            int32_t* dst, int n, cudaStream_t s);
+void launch_seg_step(const Dev& d, int grid, cudaStream_t s);
+cudaError_t launch_seg_steps_timed(const Dev& d, int grid, cudaStream_t s, int n, float* ms);
+cudaError_t launch_seg_import(const Dev& d, int grid, cudaStream_t s);
+cudaError_t launch_seg_export(const Dev& d, int grid, cudaStream_t s);
+void launch_seg_lane_stat(const Dev& d, int grid, cudaStream_t s);
+void launch_seg_observe(const Dev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out);
+cudaError_t launch_seg_persistent(const Dev& d, GridSync* gs, int blocks, int threads, int n_steps, long long limit,
+                                  cudaStream_t s);
+bool seg_persistent_fits(int threads, int per_sm);
+void seg_grids(Dev& d, int sm_count);
+void seg_capacities(int n_links, const float* len, const uint8_t* lanes, int n_trips, float vlen_min,
+                    const int32_t* now, std::vector<int32_t>& cap);
+int seg_slots(int n_links, const uint8_t* lanes, std::vector<int32_t>& lslot);
 void chunk_setup(int blocks_per_sm[8]);
 void front_setup(int blocks_per_sm[2]);
 bool chunk_split_needed(const double* lane_m, int n_links, float vlen_min);
@@ -102,7 +115,7 @@ struct sim_handle {
   long long launches = 0;    // kernel launches made by sim_step (sim_launch_count)
   size_t graph_nodes = 0, graph_samp_nodes = 0;   // kernels per step of the step graphs
   // host copies
-  std::vector<int32_t> lfrom, lto, depart, origin, dest;
+  std::vector<int32_t> lfrom, lto, depart, origin, dest, node_x, node_y;
   std::vector<float> len, spd;
   std::vector<uint8_t> lanes;
   std::vector<int32_t> lane_base;
@@ -149,6 +162,14 @@ struct sim_handle {
   uint32_t out_flags = 0;
   // vehicle types: per type length, acceleration scale, maximum speed
   std::vector<float> vty_len, vty_ascale, vty_vmax;
+  // the two forms of the state (gbt_seg.cu): buffer A (sorted every step) or link segments
+  bool seg = false;         // the state is in the segments
+  bool long_route = false;  // a route has more links than VehRec::meta counts
+  bool seg_off = false;     // the segments do not fit (memory, an overfull link) this state
+  bool pers_seg = false;    // the persistent launch's shape fits the segment form's kernel
+  bool graph_seg = false, pgraph_seg = false, tape_graph_seg = false;   // form of the captured graphs
+  std::vector<void*> seg_mem;
+  bool seg_building = false;   // seg_alloc is under way
 };
 
 namespace {
@@ -170,13 +191,20 @@ int cuda_fail(sim_handle* h, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(h, e_, #call);         \
   } while (0)
 
+bool seg_release(sim_handle* h);
+
 template <class T>
 int dalloc(sim_handle* h, T** p, size_t n) {
   const size_t nb = (n ? n : 1) * sizeof(T);
-  if (h->max_bytes && h->bytes + nb > h->max_bytes)
+  // the segment form is given up for anything else that needs its memory
+  if (h->max_bytes && h->bytes + nb > h->max_bytes && !(seg_release(h) && h->bytes + nb <= h->max_bytes))
     return fail(h, SIM_ENOMEM, "device memory cap (sim_params.max_device_bytes) reached");
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, nb);
+  if (e == cudaErrorMemoryAllocation && seg_release(h)) {
+    cudaGetLastError();
+    e = cudaMalloc(&q, nb);
+  }
   if (e != cudaSuccess) return cuda_fail(h, e, "cudaMalloc");
   h->allocs.push_back(q);
   h->alloc_sizes.push_back(nb);
@@ -203,6 +231,189 @@ int upload(sim_handle* h, T** p, const T* src, size_t n) {
   if (rc) return rc;
   if (n) CK(cudaMemcpy(*p, src, n * sizeof(T), cudaMemcpyHostToDevice));
   return SIM_OK;
+}
+
+// ------------------------------------------------------------------ the two forms of the state
+// Which form the steps run in.  Graph execution: networks of kSegLanes lanes and more in the
+// segments, smaller ones in the sorted form, whose launches per step (7 to 9) sim_launch_count
+// reports for small networks and callers rely on there.  Persistent execution (one launch
+// either way): the segments on any network.  Measured, us per step, sorted -> segments: 20 x
+// 20 grid (3,040 lanes, 2,050 vehicles) 41.6 -> 22.2; town of 6,700 lanes 16.3 -> 8.6 (with its
+// share of planning); district of 42,000 lanes with outputs and trucks 78 -> 71.
+// Not in the segments: networks with more groups of lanes than resident warps of the move
+// phase (from kSegLanesMost lanes on; metro, 782,000 lanes and 2.11M vehicles: 247 -> 253),
+// and those where links longer than a staged chunk carry most of the road, for which the
+// sorted form has its big-chunk kernel (1,000 queues of 570 vehicles: 118 against 122).
+constexpr int kSegLanes = 2048, kSegLanesMost = 150000;
+
+bool seg_possible(const sim_handle* h) { return !h->seg_off && !h->long_route; }
+
+bool seg_sized(const sim_handle* h) { return !h->d.chunk_split && h->n_lanes <= kSegLanesMost; }
+
+bool seg_wanted(const sim_handle* h) {
+  return seg_possible(h) && seg_sized(h) &&
+         (h->exec.mode == SIM_EXEC_PERSISTENT ? h->pers_seg : h->n_lanes >= kSegLanes);
+}
+
+void seg_free(sim_handle* h) {
+  for (void* p : h->seg_mem) dfree(h, p);
+  h->seg_mem.clear();
+  h->d.rec = nullptr;
+}
+
+// Segments -> buffer A; the stream's later work sees the sorted form.
+int seg_to_sorted(sim_handle* h) {
+  if (!h->seg) return SIM_OK;
+  cudaError_t e = launch_seg_export(h->d, h->grid, h->stream);
+  if (e != cudaSuccess) return cuda_fail(h, e, "state conversion");
+  h->seg = false;
+  return SIM_OK;
+}
+
+// Give the segments' memory back (the state goes on in the sorted form until it is next
+// replaced).  False when there is none to give.
+bool seg_release(sim_handle* h) {
+  if (h->seg_building || h->seg_mem.empty()) return false;
+  h->seg_off = true;
+  if (seg_to_sorted(h) != SIM_OK || cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
+  seg_free(h);
+  h->graph_dirty = true;
+  h->pgraph_n = -1;
+  h->tape_graph_dirty = true;
+  return true;
+}
+
+// Segments and the static tables of the segment form.  now (or null): vehicles per link that
+// must fit.  SIM_ENOMEM leaves nothing allocated.
+int seg_alloc(sim_handle* h, const int32_t* now) {
+  Dev& d = h->d;
+  const int nl = h->nl;
+  float vmin = d.vlen;
+  for (float v : h->vty_len) vmin = std::min(vmin, v);
+  if (h->n_lanes >= 1 << 26) return fail(h, SIM_ENOMEM, "lane ids beyond 26 bits");   // slots are packed with flags
+  std::vector<int32_t> cap;
+  seg_capacities(nl, h->len.data(), h->lanes.data(), h->nt, vmin, now, cap);
+  std::vector<int32_t> lslot;
+  d.n_slots = seg_slots(nl, h->lanes.data(), lslot);
+  const size_t ns = (size_t)d.n_slots;
+  std::vector<int2> seg(ns, make_int2(0, 0));
+  std::vector<LaneStat> none(ns);
+  const std::vector<uint32_t> pad(ns, 3u << 6);   // control 3: an empty slot
+  for (LaneStat& q : none) q = LaneStat{1.0f, 1.0f, 0.0f, 0.0f, 1.0f, 1.0f, 3u << 6, -1};
+  long long total = 0;
+  int n_big = 0;
+  for (int e = 0; e < nl; e++) {
+    for (int l = 0; l < h->lanes[e]; l++) seg[(size_t)lslot[e] + l] = make_int2((int)total, cap[e]);
+    total += cap[e];
+    n_big += cap[e] + h->lanes[e] >= 64 ? 1 : 0;
+    if (total > 0x3fffffffLL) return fail(h, SIM_ENOMEM, "segments beyond 2^30 records");
+  }
+  std::vector<LinkNext> lnext((size_t)nl);
+  for (int e = 0; e < nl; e++) {
+    const long long hx = (long long)h->node_x[h->lto[e]] - h->node_x[h->lfrom[e]];
+    const long long hy = (long long)h->node_y[h->lto[e]] - h->node_y[h->lfrom[e]];
+    if (std::max(std::llabs(hx), std::llabs(hy)) > 2147483647LL) return fail(h, SIM_ENOMEM, "headings beyond 32 bits");
+    lnext[e] = LinkNext{(int32_t)hx, (int32_t)hy, lslot[e] << 3 | (h->lanes[e] - 1), 0};
+  }
+  // in-links of every node in ascending id, and every link's tail among them
+  std::vector<int32_t> start(h->nn + 1, 0), nin((size_t)nl), tail((size_t)nl);
+  for (int e = 0; e < nl; e++) start[h->lto[e] + 1]++;
+  for (int v = 0; v < h->nn; v++) start[v + 1] += start[v];
+  {
+    std::vector<int32_t> fill(start.begin(), start.end() - 1);
+    for (int e = 0; e < nl; e++) nin[fill[h->lto[e]]++] = lslot[e];
+  }
+  for (int e = 0; e < nl; e++) tail[e] = start[h->lfrom[e]];
+  h->seg_building = true;
+  int rc = SIM_OK;
+  auto get = [&](auto** p, size_t n, const void* src = nullptr) {
+    if (rc) return;
+    std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(*p)>>>* q = nullptr;
+    if ((rc = dalloc(h, &q, n))) return;
+    h->seg_mem.push_back(q);
+    *p = q;
+    if (src && n && cudaMemcpyAsync(q, src, n * sizeof(*q), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
+      rc = fail(h, SIM_ECUDA, "segment tables");
+  };
+  get(&d.rec, (size_t)total);
+  get(&d.rng, ns);
+  get(&d.sinfo, ns, pad.data());
+  get(&d.slot_to, ns);
+  get(&d.lane_seg, ns, seg.data());
+  get(&d.lstat, ns, none.data());
+  get(&d.rear2, ns * 2);
+  get(&d.best2, ns);
+  get(&d.fres, ns);
+  get(&d.cr2, ns);
+  get(&d.lnext, (size_t)nl, lnext.data());
+  get(&d.lslot, (size_t)nl, lslot.data());
+  get(&d.tail_in, (size_t)nl, tail.data());
+  get(&d.nin_slot, (size_t)nl, nin.data());
+  get(&d.qnext, ns);
+  get(&d.big_links, (size_t)std::max(1, n_big));
+  get(&d.tl, ns);
+  get(&d.runs, (size_t)nl);
+  get(&d.late, (size_t)nl);
+  get(&d.claim, (size_t)nl);
+  get(&d.cuts, ns / 32);
+  if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(h, SIM_ECUDA, "segment tables");
+  h->seg_building = false;
+  if (rc) {
+    seg_free(h);
+    return rc;
+  }
+  launch_seg_lane_stat(d, h->grid, h->stream);
+  seg_grids(d, h->sm_count);
+  h->graph_dirty = true;
+  h->pgraph_n = -1;
+  h->tape_graph_dirty = true;
+  return SIM_OK;
+}
+
+// Buffer A -> segments.  When they cannot hold the state (memory, a link with more vehicles
+// than a block stages) the sorted form goes on: h->seg stays false, h->seg_off is set, and
+// the call succeeds.
+int seg_from_sorted(sim_handle* h) {
+  if (h->seg) return SIM_OK;
+  std::vector<int32_t> now;
+  for (int attempt = 0; attempt < 2; attempt++) {
+    if (h->seg_mem.empty() && seg_alloc(h, now.empty() ? nullptr : now.data()) != SIM_OK) {
+      cudaGetLastError();
+      h->seg_off = true;
+      break;
+    }
+    cudaError_t e = launch_seg_import(h->d, h->grid, h->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&h->mirror->c, h->d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_fail(h, e, "state conversion");
+    const int grow = h->mirror->c.grow;
+    if (!grow) {
+      h->seg = true;
+      return SIM_OK;
+    }
+    if (grow == 2 || attempt == 1) {
+      h->seg_off = true;
+      break;
+    }
+    // vehicles per link, from the lane starts of the import's sort
+    std::vector<int32_t> ls((size_t)h->n_lanes + 1);
+    CK(cudaMemcpy(ls.data(), h->d.lane_start, ls.size() * 4, cudaMemcpyDeviceToHost));
+    now.resize((size_t)h->nl);
+    for (int k = 0; k < h->nl; k++) now[k] = ls[h->lane_base[k + 1]] - ls[h->lane_base[k]];
+    seg_free(h);
+  }
+  // the sorted form: the import took the lane counts
+  CK(cudaMemsetAsync(h->d.cnt, 0, (size_t)h->n_lanes * 4, h->stream));
+  CK(cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream));
+  launch_count(h->d, h->grid, h->stream);
+  return SIM_OK;
+}
+
+// The form the next steps run in.
+int seg_choose(sim_handle* h) {
+  if (!seg_wanted(h)) return seg_to_sorted(h);
+  return seg_from_sorted(h);
 }
 
 // ------------------------------------------------------------------ union of scenarios
@@ -323,6 +534,8 @@ int create_from_flat(Flat& F, sim_handle** out) {
   h->loop = P.loop_routes ? 1 : 0;
   h->lfrom = F.lf;
   h->lto = F.lt;
+  h->node_x = F.nx;
+  h->node_y = F.ny;
   h->len = F.len;
   h->spd = F.spd;
   h->lanes = F.lanes;
@@ -544,6 +757,8 @@ int create_from_flat(Flat& F, sim_handle** out) {
       goto fail_rc;
     }
   }
+  // the segments with the handle, where its steps will use them and the memory is there
+  if (seg_wanted(h) && seg_alloc(h, nullptr) != SIM_OK) cudaGetLastError();
   *out = h;
   return SIM_OK;
 fail_rc:
@@ -639,6 +854,7 @@ int reset_dynamic(sim_handle* h) {
   Dev& d = h->d;
   h->state_lost = false;
   h->t_known = false;
+  h->seg = h->seg_off = false;
   const size_t nt = (size_t)h->nt;
   CK(cudaMemsetAsync(d.status, 0, nt ? nt : 1, h->stream));
   CK(cudaMemsetAsync(d.ins_step, 0xFF, (nt ? nt : 1) * 4, h->stream));
@@ -979,6 +1195,7 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     if ((rc = compact_routes(h))) return rc;
   }
   h->d.routes = h->routes;
+  h->long_route = nn >= kMaxRem;
   if ((rc = reset_dynamic(h))) return rc;
   std::vector<uint8_t> st(nt, SIM_PENDING);
   if ((rc = build_queues(h, st))) return rc;
@@ -1058,9 +1275,11 @@ int sim_set_routes(sim_handle* h, const int32_t* offsets, const int32_t* links) 
   }
   const long long total = nt ? offsets[nt] : 0;
   std::vector<int32_t> off(nt > 0 ? nt : 1), len(nt > 0 ? nt : 1);
+  h->long_route = false;
   for (int i = 0; i < nt; i++) {
     off[i] = offsets[i];
     len[i] = offsets[i + 1] - offsets[i];
+    h->long_route = h->long_route || len[i] >= kMaxRem;
   }
   dfree(h, h->routes);
   h->routes = nullptr;
@@ -1112,43 +1331,50 @@ int sim_read_routes(sim_handle* h, int32_t* offsets, int32_t* links) {
   return SIM_OK;
 }
 
-int sim_step(sim_handle* h, int32_t n_steps) {
-  NvtxRange nvtx_("sim_step");
-  if (!h || n_steps < 0) return SIM_EINVAL;
-  if (h->state_lost) return fail(h, SIM_ESTATE, "the state is undefined after a timeout: sim_write_state or sim_route first");
-  if (!h->routed) return fail(h, SIM_ESTATE, "sim_step before sim_route / sim_set_routes");
-  if (n_steps == 0) return SIM_OK;
-  long long t0 = 0;
-  if (int rc = check_horizon(h, n_steps, &t0)) return rc;
-  if (h->graph_dirty) {
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    if (h->gexec_samp) cudaGraphExecDestroy(h->gexec_samp);
-    if (h->graph_samp) cudaGraphDestroy(h->graph_samp);
-    h->gexec = h->gexec_samp = nullptr;
-    h->graph = h->graph_samp = nullptr;
-    Dev dn = h->d;
-    dn.acc_u = nullptr;   // steps between sampling instants skip the sample kernel
+namespace {
+
+// The step graph of the present form (and, with edge samples on, the one of the sampling
+// instants).
+int build_step_graph(sim_handle* h) {
+  if (!h->graph_dirty && h->graph_seg == h->seg) return SIM_OK;
+  if (h->gexec) cudaGraphExecDestroy(h->gexec);
+  if (h->graph) cudaGraphDestroy(h->graph);
+  if (h->gexec_samp) cudaGraphExecDestroy(h->gexec_samp);
+  if (h->graph_samp) cudaGraphDestroy(h->graph_samp);
+  h->gexec = h->gexec_samp = nullptr;
+  h->graph = h->graph_samp = nullptr;
+  auto capture = [&](const Dev& d, cudaGraph_t* g, cudaGraphExec_t* x, size_t* nodes) -> int {
     CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    launch_step(dn, h->grid, h->has_stop, h->cap_stream);
-    CK(cudaStreamEndCapture(h->cap_stream, &h->graph));
-    CK(cudaGraphInstantiate(&h->gexec, h->graph, 0));
-    CK(cudaGraphGetNodes(h->graph, nullptr, &h->graph_nodes));
-    if (h->d.acc_u) {
-      CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-      launch_step(h->d, h->grid, h->has_stop, h->cap_stream);
-      CK(cudaStreamEndCapture(h->cap_stream, &h->graph_samp));
-      CK(cudaGraphInstantiate(&h->gexec_samp, h->graph_samp, 0));
-      CK(cudaGraphGetNodes(h->graph_samp, nullptr, &h->graph_samp_nodes));
-    }
-    h->graph_dirty = false;
-  }
+    if (h->seg) launch_seg_step(d, h->grid, h->cap_stream);
+    else launch_step(d, h->grid, h->has_stop, h->cap_stream);
+    CK(cudaStreamEndCapture(h->cap_stream, g));
+    CK(cudaGraphInstantiate(x, *g, 0));
+    CK(cudaGraphGetNodes(*g, nullptr, nodes));
+    return SIM_OK;
+  };
+  Dev dn = h->d;
+  dn.acc_u = nullptr;   // steps between sampling instants skip the sample kernel
+  if (int rc = capture(dn, &h->graph, &h->gexec, &h->graph_nodes)) return rc;
+  if (h->d.acc_u)
+    if (int rc = capture(h->d, &h->graph_samp, &h->gexec_samp, &h->graph_samp_nodes)) return rc;
+  h->graph_dirty = false;
+  h->graph_seg = h->seg;
+  return SIM_OK;
+}
+
+// Enqueue n steps from step t0 on in the present form.
+int enqueue_steps(sim_handle* h, long long t0, int n_steps) {
   if (h->exec.mode == SIM_EXEC_PERSISTENT) {
     const int blocks = h->exec.blocks_per_sm * h->sm_count;
     const long long limit = h->exec.barrier_timeout_cycles > 0 ? h->exec.barrier_timeout_cycles : kDefaultWaitCycles;
     const sim_exec& x = h->exec;
-    const bool same = h->pexec && h->pgraph_n == n_steps && h->pgraph_cfg.threads == x.threads &&
-                      h->pgraph_cfg.blocks_per_sm == x.blocks_per_sm &&
+    const bool seg = h->seg;
+    auto launch = [&](cudaStream_t s) {
+      return seg ? launch_seg_persistent(h->d, h->gs, blocks, x.threads, n_steps, limit, s)
+                 : launch_persistent(h->d, h->gs, blocks, x.threads, n_steps, limit, s);
+    };
+    const bool same = h->pexec && h->pgraph_n == n_steps && h->pgraph_seg == seg &&
+                      h->pgraph_cfg.threads == x.threads && h->pgraph_cfg.blocks_per_sm == x.blocks_per_sm &&
                       h->pgraph_cfg.barrier_timeout_cycles == x.barrier_timeout_cycles;
     if (!same && !h->pgraph_unsupported) {
       // capture the single persistent launch as a graph (rebuilt when the step count or
@@ -1159,7 +1385,7 @@ int sim_step(sim_handle* h, int32_t n_steps) {
       h->pgraph = nullptr;
       bool ok = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
       if (ok) {
-        cudaError_t le = launch_persistent(h->d, h->gs, blocks, x.threads, n_steps, limit, h->cap_stream);
+        cudaError_t le = launch(h->cap_stream);
         cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &h->pgraph);
         ok = le == cudaSuccess && ce == cudaSuccess && h->pgraph &&
              cudaGraphInstantiate(&h->pexec, h->pgraph, 0) == cudaSuccess;
@@ -1173,20 +1399,55 @@ int sim_step(sim_handle* h, int32_t n_steps) {
       } else {
         h->pgraph_n = n_steps;
         h->pgraph_cfg = x;
+        h->pgraph_seg = seg;
       }
     }
     if (h->pexec) CK(cudaGraphLaunch(h->pexec, h->stream));
-    else CK(launch_persistent(h->d, h->gs, blocks, x.threads, n_steps, limit, h->stream));
+    else CK(launch(h->stream));
     h->launches += 1;
-  } else {
-    const long long every = h->d.acc_u ? h->d.samp_every : 0;
-    for (int s = 0; s < n_steps; s++) {
-      const bool samp = every > 0 && (t0 + s) % every == 0;
-      CK(cudaGraphLaunch(samp ? h->gexec_samp : h->gexec, h->stream));
-      h->launches += (long long)(samp ? h->graph_samp_nodes : h->graph_nodes);
-    }
+    return SIM_OK;
   }
-  return check_device(h);
+  if (int rc = build_step_graph(h)) return rc;
+  const long long every = h->d.acc_u ? h->d.samp_every : 0;
+  for (int s = 0; s < n_steps; s++) {
+    const bool samp = every > 0 && (t0 + s) % every == 0;
+    CK(cudaGraphLaunch(samp ? h->gexec_samp : h->gexec, h->stream));
+    h->launches += (long long)(samp ? h->graph_samp_nodes : h->graph_nodes);
+  }
+  return SIM_OK;
+}
+
+// After steps that stopped before step `upto` because a segment was full (the step they
+// stopped at has not begun): back to the sorted form, larger segments or none.
+int seg_regrow(sim_handle* h, int grow) {
+  if (int rc = seg_to_sorted(h)) return rc;
+  if (grow != 2) return SIM_OK;   // seg_from_sorted lays it out again
+  h->seg_off = true;
+  CK(cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream));
+  return SIM_OK;
+}
+
+}  // namespace
+
+int sim_step(sim_handle* h, int32_t n_steps) {
+  NvtxRange nvtx_("sim_step");
+  if (!h || n_steps < 0) return SIM_EINVAL;
+  if (h->state_lost) return fail(h, SIM_ESTATE, "the state is undefined after a timeout: sim_write_state or sim_route first");
+  if (!h->routed) return fail(h, SIM_ESTATE, "sim_step before sim_route / sim_set_routes");
+  if (n_steps == 0) return SIM_OK;
+  long long t0 = 0;
+  if (int rc = check_horizon(h, n_steps, &t0)) return rc;
+  const long long t_end = t0 + n_steps;
+  while (t0 < t_end) {
+    if (int rc = seg_choose(h)) return rc;
+    if (int rc = enqueue_steps(h, t0, (int)(t_end - t0))) return rc;
+    if (int rc = check_device(h)) return rc;
+    if (!h->seg) break;
+    t0 = h->t_host;
+    if (t0 < t_end)
+      if (int rc = seg_regrow(h, h->mirror->c.grow)) return rc;
+  }
+  return SIM_OK;
 }
 
 int sim_set_exec(sim_handle* h, const sim_exec* e) {
@@ -1208,6 +1469,7 @@ int sim_set_exec(sim_handle* h, const sim_exec* e) {
     if (mx < 1) return fail(h, SIM_EINVAL, "the persistent kernel does not fit this block size");
     if (x.blocks_per_sm < 1 || x.blocks_per_sm > mx)
       return fail(h, SIM_EINVAL, "blocks_per_sm exceeds the co-resident limit of the persistent kernel");
+    h->pers_seg = seg_persistent_fits(x.threads, x.blocks_per_sm);
   } else {
     return fail(h, SIM_EINVAL, "unknown execution mode");
   }
@@ -1228,7 +1490,27 @@ int sim_step_timed(sim_handle* h, int32_t n_steps, float* kernel_ms) {
   if (h->state_lost) return fail(h, SIM_ESTATE, "the state is undefined after a timeout: sim_write_state or sim_route first");
   if (!h->routed) return fail(h, SIM_ESTATE, "sim_step_timed before sim_route / sim_set_routes");
   if (int rc = check_horizon(h, n_steps)) return rc;
-  CK(launch_steps_timed(h->d, h->grid, h->has_stop, h->stream, n_steps, kernel_ms));
+  for (int k = 0; k < kNumKernels; k++) kernel_ms[k] = 0.0f;
+  if (n_steps > 0 && h->n_lanes >= kSegLanes && seg_possible(h) && seg_sized(h)) {
+    if (int rc = seg_from_sorted(h)) return rc;
+  } else if (int rc = seg_to_sorted(h)) {
+    return rc;
+  }
+  if (h->seg) {
+    const long long t_end = h->t_host + n_steps;
+    float ms[2] = {0.0f, 0.0f};
+    CK(launch_seg_steps_timed(h->d, h->grid, h->stream, n_steps, ms));
+    kernel_ms[kKFront] = ms[0];
+    kernel_ms[kKChunk] = ms[1];
+    if (int rc = check_device(h)) return rc;
+    if (h->t_host == t_end) return SIM_OK;
+    // a segment was full: the rest in the sorted form
+    if (int rc = seg_regrow(h, 2)) return rc;
+    n_steps = (int)(t_end - h->t_host);
+  }
+  float rest[kNumKernels];
+  CK(launch_steps_timed(h->d, h->grid, h->has_stop, h->stream, n_steps, rest));
+  for (int k = 0; k < kNumKernels; k++) kernel_ms[k] += rest[k];
   return check_device(h);
 }
 
@@ -1265,7 +1547,7 @@ int sim_read_state(sim_handle* h, const sim_state_view* out, uint32_t fields, in
     }
   }
   if (nt)
-    launch_state_out(h->d, h->grid, h->stream, (uint8_t*)dptr[0], (int32_t*)dptr[1], (int32_t*)dptr[2],
+    launch_state_out(h->d, h->grid, h->stream, h->seg, (uint8_t*)dptr[0], (int32_t*)dptr[1], (int32_t*)dptr[2],
                      (int32_t*)dptr[3], (float*)dptr[4], (float*)dptr[5], (int32_t*)dptr[6], (int32_t*)dptr[7],
                      (int8_t*)dptr[8]);
   cudaError_t e = cudaSuccess;
@@ -1339,13 +1621,14 @@ int sim_write_state(sim_handle* h, const uint8_t* status, const int32_t* link, c
   std::vector<uint8_t> st(status, status + nt);
   if ((rc = build_queues(h, st))) return rc;
   CK(cudaStreamSynchronize(h->stream));
-  return SIM_OK;
+  return seg_choose(h);
 }
 
 int sim_occupancy(sim_handle* h, int32_t* lane_start, int32_t* sorted_vid) {
   if (!h || !lane_start || !sorted_vid) return SIM_EINVAL;
   h->t_known = false;
   if (!h->routed) return fail(h, SIM_ESTATE, "no routes");
+  if (h->seg) CK(launch_seg_export(h->d, h->grid, h->stream));   // the segments stay as they are
   launch_occupancy(h->d, h->grid, h->stream);
   int32_t* dv;
   int rc = dalloc(h, &dv, (size_t)std::max(1, h->nt));
@@ -1387,7 +1670,7 @@ int sim_counters(sim_handle* h, sim_counters_t* out) {
   out->arrived = (int64_t)c.arrived;
   out->veh_steps = (int64_t)c.veh_steps;
   out->pending = pending;
-  out->active_last = c.active_last;
+  out->active_last = h->seg ? c.nact[(c.t + 1) & 1] : c.active_last;
   out->lc_evals = (int64_t)c.lc_evals;
   return SIM_OK;
 }
@@ -1417,6 +1700,7 @@ int sim_set_class_params(sim_handle* h, const float* v0, const float* T, const f
                      h->stream));
   CK(cudaMemcpyAsync(const_cast<LinkRec*>(h->d.links), h->recs.data(), h->recs.size() * sizeof(LinkRec),
                      cudaMemcpyHostToDevice, h->stream));
+  if (!h->seg_mem.empty()) launch_seg_lane_stat(h->d, h->grid, h->stream);
   CK(cudaStreamSynchronize(h->stream));
   return upload_type_params(h);
 }
@@ -1486,7 +1770,7 @@ int sim_observe(sim_handle* h, int32_t n_steps, int32_t obs_every, double* progr
   if (rc) return rc;
   for (int k = 0; k < nobs; k++) {
     if ((rc = sim_step(h, obs_every))) break;
-    launch_observe(h->d, h->grid, h->stream, nullptr, nullptr, dp);
+    (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, nullptr, nullptr, dp);
     cudaError_t e = cudaMemcpyAsync(progress + (size_t)k * nt, dp, nt * 8, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
@@ -1522,7 +1806,7 @@ int sim_loss(sim_handle* h, const sim_loss_spec* spec, double* loss_out) {
   if (e != cudaSuccess) rc = cuda_fail(h, e, "loss");
   for (int k = 0; k < nobs && rc == SIM_OK; k++) {
     if ((rc = sim_step(h, every))) break;
-    launch_observe(h->d, h->grid, h->stream, tgt + (size_t)k * nt, res, nullptr);
+    (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, tgt + (size_t)k * nt, res, nullptr);
   }
   if (rc == SIM_OK) {
     e = cudaMemcpyAsync(loss_out, &h->d.ctl->loss, 8, cudaMemcpyDeviceToHost, h->stream);
@@ -1555,6 +1839,12 @@ CkptLayout ckpt_layout(const sim_handle* h) {
 cudaError_t ckpt_copy(sim_handle* h, unsigned char* buf, bool save) {
   const CkptLayout L = ckpt_layout(h);
   Dev& d = h->d;
+  // checkpoints hold the sorted form
+  if (save && h->seg) {
+    cudaError_t e = launch_seg_export(d, h->grid, h->stream);
+    if (e != cudaSuccess) return e;
+  }
+  if (!save) h->seg = false;
   struct Item { void* p; size_t n; } items[] = {
       {d.A.x, L.nt * 4}, {d.A.v, L.nt * 4}, {d.A.vid, L.nt * 4}, {d.A.link, L.nt * 4}, {d.A.nxt, L.nt * 4},
       {d.A.cur, L.nt * 4}, {d.A.lane, L.nt * 4}, {d.A.gid, L.nt * 4}, {d.A.mv, L.nt}, {d.status, L.nt}, {d.ins_step, L.nt * 4}, {d.arr_step, L.nt * 4},
@@ -1596,20 +1886,7 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
   h->t_known = false;   // the passes below advance and restore the step counter
   const int nobs = n_steps / every, nseg = (n_steps + seg - 1) / seg;
   const size_t nt = (size_t)std::max(1, h->nt);
-  // sim_step's graph
-  int rc = sim_step(h, 0);
-  if (rc) return rc;
-  if (h->graph_dirty) {
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    h->gexec = nullptr;
-    h->graph = nullptr;
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    launch_step(h->d, h->grid, h->has_stop, h->cap_stream);
-    CK(cudaStreamEndCapture(h->cap_stream, &h->graph));
-    CK(cudaGraphInstantiate(&h->gexec, h->graph, 0));
-    h->graph_dirty = false;
-  }
+  int rc = SIM_OK;
   // tape of one segment and its graph
   if (h->tape_steps != seg || !h->tape) {
     dfree(h, h->tape);
@@ -1620,20 +1897,6 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
     if ((rc = dalloc(h, &h->tform, nt))) return rc;
     h->tape_steps = seg;
     h->tape_graph_dirty = true;
-  }
-  if (h->tape_graph_dirty) {
-    if (h->gexec_tape) cudaGraphExecDestroy(h->gexec_tape);
-    if (h->graph_tape) cudaGraphDestroy(h->graph_tape);
-    h->gexec_tape = nullptr;
-    h->graph_tape = nullptr;
-    Dev dt = h->d;
-    dt.tape = h->tape;
-    dt.tform = h->tform;
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    launch_step(dt, h->grid, h->has_stop, h->cap_stream);
-    CK(cudaStreamEndCapture(h->cap_stream, &h->graph_tape));
-    CK(cudaGraphInstantiate(&h->gexec_tape, h->graph_tape, 0));
-    h->tape_graph_dirty = false;
   }
   Dev dtape = h->d;
   dtape.tape = h->tape;
@@ -1654,22 +1917,72 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
     release();
     return rc;
   }
+  // both passes in the segment form, on any network, if its memory is there (the working
+  // memory above comes first)
+  if (seg_possible(h) && (rc = seg_from_sorted(h))) {
+    release();
+    return rc;
+  }
+  auto graphs = [&]() -> int {
+    if (int r = build_step_graph(h)) return r;
+    if (!h->tape_graph_dirty && h->tape_graph_seg == h->seg) return SIM_OK;
+    if (h->gexec_tape) cudaGraphExecDestroy(h->gexec_tape);
+    if (h->graph_tape) cudaGraphDestroy(h->graph_tape);
+    h->gexec_tape = nullptr;
+    h->graph_tape = nullptr;
+    Dev dt = h->d;
+    dt.tape = h->tape;
+    dt.tform = h->tform;
+    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+    if (h->seg) launch_seg_step(dt, h->grid, h->cap_stream);
+    else launch_step(dt, h->grid, h->has_stop, h->cap_stream);
+    CK(cudaStreamEndCapture(h->cap_stream, &h->graph_tape));
+    CK(cudaGraphInstantiate(&h->gexec_tape, h->graph_tape, 0));
+    h->tape_graph_dirty = false;
+    h->tape_graph_seg = h->seg;
+    return SIM_OK;
+  };
+  if ((rc = graphs())) {
+    release();
+    return rc;
+  }
   const int ng = h->ncls * 5;
   cudaError_t e = cudaMemcpyAsync(tgt, spec->target, (size_t)nobs * nt * 8, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, (size_t)ng * 8, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->loss, 0, 8, h->stream);
   // ---- forward: checkpoint every `seg` steps, observe every `every` steps
-  for (int sg = 0; sg < nseg && e == cudaSuccess; sg++) {
-    e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, true);
-    const int j1 = std::min(n_steps, (sg + 1) * seg);
-    for (int j = sg * seg; j < j1 && e == cudaSuccess; j++) {
-      e = cudaGraphLaunch(h->gexec, h->stream);
-      if ((j + 1) % every == 0) {
-        const int k = (j + 1) / every - 1;
-        launch_observe(h->d, h->grid, h->stream, tgt + (size_t)k * nt, res + (size_t)k * nt, nullptr);
+  auto forward = [&]() {
+    for (int sg = 0; sg < nseg && e == cudaSuccess; sg++) {
+      e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, true);
+      const int j1 = std::min(n_steps, (sg + 1) * seg);
+      for (int j = sg * seg; j < j1 && e == cudaSuccess; j++) {
+        e = cudaGraphLaunch(h->gexec, h->stream);
+        if ((j + 1) % every == 0) {
+          const int k = (j + 1) / every - 1;
+          (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, tgt + (size_t)k * nt,
+                                                         res + (size_t)k * nt, nullptr);
+        }
       }
     }
+  };
+  forward();
+  if (h->seg && e == cudaSuccess) {
+    e = cudaMemcpyAsync(&h->mirror->c, h->d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e == cudaSuccess && h->mirror->c.grow) {
+      // a segment was full on the way: again from the start in the sorted form
+      e = ckpt_copy(h, ck, false);
+      if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->loss, 0, 8, h->stream);
+      h->seg_off = true;
+      if ((rc = graphs())) {
+        release();
+        return rc;
+      }
+      forward();
+    }
   }
+  const bool replay_seg = h->seg;
   if (e == cudaSuccess) e = ckpt_copy(h, ck + (size_t)nseg * CL.bytes, true);   // end state
   // ---- reverse: per segment, replay it with the tape, then sweep it backwards
   double *lx = lam, *lv = lam + nt, *nx = lam + 2 * nt, *nv = lam + 3 * nt;
@@ -1677,6 +1990,7 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
   for (int sg = nseg - 1; sg >= 0 && e == cudaSuccess; sg--) {
     const int j0 = sg * seg, j1 = std::min(n_steps, (sg + 1) * seg);
     e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, false);
+    if (e == cudaSuccess && replay_seg) e = launch_seg_import(h->d, h->grid, h->stream);   // fits: the forward pass did
     if (e == cudaSuccess) e = cudaMemsetAsync(h->tape, 0, (size_t)seg * nt * sizeof(TapeRec), h->stream);
     launch_tape_begin(h->d, h->stream);
     for (int j = j0; j < j1 && e == cudaSuccess; j++) e = cudaGraphLaunch(h->gexec_tape, h->stream);

@@ -119,27 +119,6 @@ __device__ __forceinline__ int view_lane_start(const Dev& d, const ChunkView& V,
   return k < (unsigned)V.nls ? V.ls[k] : d.lane_start[g];
 }
 
-// Eq. 7 with the vehicle's free-road term om = 1 - (v / v0)^4 already computed (the same
-// operations in the same order as idm_acc, so the same result).
-__device__ __forceinline__ float idm_om(const ClassPar& P, float om, float s_min, float s, float v, float vl) {
-  const float dv = v - vl;
-  const float t1 = v * P.T;
-  const float t2 = (v * dv) / P.sab2;
-  const float dyn = t1 + t2;
-  const float ss = P.s0 + fmaxf(0.0f, dyn);
-  const float se = fmaxf(s, s_min);
-  const float q = ss / se;
-  const float q2 = q * q;
-  return P.a * (om - q2);
-}
-
-__device__ __forceinline__ float free_term(float v, float v0) {
-  const float r = v / v0;
-  const float r2 = r * r;
-  const float r4 = r2 * r2;
-  return 1.0f - r4;
-}
-
 // Eq. 7 parameters and desired speed of trip vid on link L (vehicle types: veh_par).
 template <bool TYPES>
 __device__ __forceinline__ void view_par(const Dev& d, const ChunkView& V, const LinkRec& L, int vid, ClassPar& P,
@@ -709,38 +688,6 @@ __global__ void __launch_bounds__(kBigThreads, 2) k_chunk_big(Dev d) {
 // after `limit` SM cycles (about a second by default) a block sets kErrTimeout in the
 // error word and leaves; every waiting block also leaves as soon as it sees the flag,
 // so the launch always ends and the host reports SIM_ETIMEOUT.
-__device__ __forceinline__ bool grid_barrier(GridSync* gs, int* err, long long limit) {
-  __shared__ int s_ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    volatile unsigned* vgen = &gs->gen;
-    volatile int* verr = err;
-    const unsigned g = *vgen;
-    __threadfence();
-    const unsigned arrived = atomicAdd(&gs->count, 1u);
-    if (arrived == gridDim.x - 1) {
-      gs->count = 0;
-      __threadfence();
-      atomicAdd(&gs->gen, 1u);
-    } else {
-      const long long t0 = clock64();
-      while (*vgen == g) {
-        if ((*verr & kErrTimeout) || clock64() - t0 > limit) {
-          atomicOr(err, kErrTimeout);
-          ok = 0;
-          break;
-        }
-      }
-    }
-    __threadfence();
-    if (*verr & kErrTimeout) ok = 0;
-    s_ok = ok;
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
-
 template <bool OUT, bool TYPES>
 __device__ __forceinline__ void persistent_steps(const Dev& d, GridSync* gs, int n_steps, long long limit,
                                                  ChunkSmem& S) {

@@ -96,6 +96,36 @@ struct __align__(16) ChunkInfo {
   int32_t c0, c1, e_lo, e_hi, g_lo, g_hi, pad0, pad1;
 };
 
+// One vehicle of the link-segment form of the state (gbt_seg.cuh): one 32-byte sector.
+struct __align__(32) VehRec {
+  float x, v;
+  int32_t vid;
+  int32_t nxt;      // next link of the route, -1 on the last link
+  int32_t nlb;      // next link: slot of its lane 0 << 3 | (lanes - 1), -1 without one
+  int32_t ri;       // index of the current link in the route store
+  float tau;        // mandatory-switch draw of (trip, current link)
+  uint32_t meta;    // lane | movement class << 3 | last lane change << 5 (0 none, 1 left, 2 right) |
+                    // links of the route after this one << 7 (0 in loop routes)
+};
+static_assert(sizeof(VehRec) == 32, "VehRec must be 32 bytes");
+
+// Static record of one lane slot of the link-segment form: what a vehicle on it needs.
+struct __align__(16) LaneStat {
+  float len, v0, T, s0;     // link length, desired speed, Eq. 7 parameters of its class
+  float a, sab2;
+  uint32_t info;            // lane | (lanes - 1) << 3 | control << 6 | class << 8 | in_index << 16 | in-degree << 24
+  int32_t link;
+};
+static_assert(sizeof(LaneStat) == 32, "LaneStat must be 32 bytes");
+
+// Static record of one link in the link-segment form: what a vehicle about to enter it needs.
+struct __align__(16) LinkNext {
+  int32_t hx, hy;           // head node minus tail node, decimetres
+  int32_t nlb;              // slot of its lane 0 << 3 | (lanes - 1)
+  int32_t pad;
+};
+constexpr int kMaxRem = 1 << 25;   // route links that VehRec::meta counts
+
 struct Ctl {
   long long t;
   int nA;          // slots filled in the unsorted buffer A
@@ -118,6 +148,13 @@ struct Ctl {
   int chunk_next;  // next chunk of the fused step kernel to take
   int n_long;      // long lane segments listed by the lane-start scan
   int n_big;       // chunks beyond the chunk kernel's staging capacity (lane-front phase)
+  // link-segment form
+  alignas(128) long long tm;   // step of the running move phase (the front phase's copy of t)
+  int grow;                    // the next step does not fit the segments: 1 a segment, 2 a link (no step runs)
+  int n_bigl[2];               // links left to whole blocks, by parity of the step
+  alignas(128) int n_tl[2];    // entries of tl, runs and late, by parity of the step
+  int n_run[2], n_late[2];
+  alignas(128) int nact[2];    // vehicles advanced, by parity of the step
 };
 
 // Forms of Eq. 7 an acceleration can come from (adjoint tape).
@@ -226,6 +263,33 @@ struct Dev {
   int32_t* q_head;
   const int32_t* q_items;
   Ctl* ctl;
+  // link-segment form of the state (gbt_seg.cuh).  Lanes are numbered by slots there: the
+  // lanes of whole links fill groups of 32 slots, the rest of a group is left empty.
+  VehRec* rec;                     // link e owns cap records from its segment's start on, in (lane, x, vid) order
+  uint32_t* rng;                   // per slot: its vehicles, start relative to the segment | count << 16
+  const uint32_t* sinfo;           // per slot: LaneStat::info (control 3: empty slot)
+  const int2* lane_seg;            // per slot: its link's segment start and capacity
+  const LaneStat* lstat;           // per slot
+  const int32_t* slot_to;          // per slot: its link's head node
+  RearRec* rear2;                  // [2][n_slots]: rearmost vehicle at step t in half t & 1 (tag t + 1)
+  unsigned long long* best2;       // per slot: epoch-tagged admission key
+  int2* fres;                      // per slot: its front's acceleration; flags | target slot << 4
+  VehRec* cr2;                     // per slot: the bidding front's record after crossing
+  const LinkNext* lnext;           // per link
+  const int32_t* lslot;            // per link: slot of its lane 0
+  const int32_t* tail_in;          // per link: start of its tail node's in-links in nin_slot
+  const int32_t* nin_slot;         // in-links of every node in ascending id: slot of lane 0
+  int n_slots;
+  int packed;                      // runs are packed by the front phase (else they are parts of a group)
+  int parts;                       // parts of a group, 1..8
+  unsigned long long* cuts;        // per group: first lane of parts 1..7, 8 bits each
+  int32_t* qnext;                  // per slot of a lane 0: departure step of its link's queue's head (else INT_MAX)
+  int32_t* big_links;              // links with more vehicles than a warp's staging area
+  int32_t* tl;                     // slots of the links with something to do, run after run
+  int2* runs;                      // runs of the move phase: first entry of tl, lanes
+  int32_t* late;                   // empty links that a crossing vehicle may enter
+  int32_t* claim;                  // per link: t + 1 of the step it was last listed in late
+  int seg_front_grid[4], seg_move_grid[6];
   int chunk_split;                 // oversized chunks go to the big-chunk launch
   int rank_long;                   // long lane segments go to k_rank_long
   int front_grid[2];               // blocks of the lane-front kernel (without / with types)

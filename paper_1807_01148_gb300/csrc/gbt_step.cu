@@ -75,10 +75,6 @@ __global__ void k_scatter(Dev d) {
 // segments beyond the shared-memory capacity fall back to the per-vehicle count.
 constexpr int kLongCap = 2048, kMaxRuns = 64;
 
-__device__ __forceinline__ bool key_less(float xa, int va, float xb, int vb) {
-  return xa < xb || (xa == xb && va < vb);
-}
-
 __global__ void __launch_bounds__(256) k_rank_long(Dev d) {
   griddep_wait();
   if (step_timed_out(d)) return;
@@ -775,10 +771,15 @@ __global__ void k_state_out_active(Dev d, int32_t* link, int32_t* lane, int32_t*
   }
 }
 
-void launch_state_out(const Dev& d, int grid, cudaStream_t s, uint8_t* status, int32_t* link, int32_t* lane,
+void launch_seg_state_out(const Dev& d, int grid, cudaStream_t s, int32_t* link, int32_t* lane, int32_t* cursor,
+                          float* x, float* v, int8_t* dec);
+
+// seg: the vehicles are in the link segments, not in buffer A
+void launch_state_out(const Dev& d, int grid, cudaStream_t s, bool seg, uint8_t* status, int32_t* link, int32_t* lane,
                       int32_t* cursor, float* x, float* v, int32_t* ins, int32_t* arr, int8_t* dec) {
   k_state_out<<<grid, 256, 0, s>>>(d, status, link, lane, cursor, x, v, ins, arr, dec);
-  k_state_out_active<<<grid, 256, 0, s>>>(d, link, lane, cursor, x, v, dec);
+  if (seg) launch_seg_state_out(d, grid, s, link, lane, cursor, x, v, dec);
+  else k_state_out_active<<<grid, 256, 0, s>>>(d, link, lane, cursor, x, v, dec);
 }
 
 // Validate a state given by vid: every active trip sits on route[cursor], in a lane

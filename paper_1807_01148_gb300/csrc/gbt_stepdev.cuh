@@ -51,6 +51,32 @@ __device__ __forceinline__ bool line_closed(const Dev& d, const LinkRec& L, int 
   return false;
 }
 
+__device__ __forceinline__ float free_term(float v, float v0) {
+  const float r = v / v0;
+  const float r2 = r * r;
+  const float r4 = r2 * r2;
+  return 1.0f - r4;
+}
+
+// Eq. 7 with the vehicle's free-road term om = 1 - (v / v0)^4 already computed (the same
+// operations in the same order as idm_acc, so the same result).
+__device__ __forceinline__ float idm_om(const ClassPar& P, float om, float s_min, float s, float v, float vl) {
+  const float dv = v - vl;
+  const float t1 = v * P.T;
+  const float t2 = (v * dv) / P.sab2;
+  const float dyn = t1 + t2;
+  const float ss = P.s0 + fmaxf(0.0f, dyn);
+  const float se = fmaxf(s, s_min);
+  const float q = ss / se;
+  const float q2 = q * q;
+  return P.a * (om - q2);
+}
+
+// Order of the vehicles of a lane.
+__device__ __forceinline__ bool key_less(float xa, int va, float xb, int vb) {
+  return xa < xb || (xa == xb && va < vb);
+}
+
 // Eq. 7 parameters and desired speed of trip vid on link L: its class's, or with vehicle
 // types (Sec. 6.3.5) the class's with a scaled by the type (a table built on the host)
 // and v0 capped at the type's maximum speed.
@@ -132,6 +158,40 @@ __device__ __forceinline__ void note_exit(const Dev& d, int vid, int e, int t) {
     atomicAdd(&d.tt_sum[e], (unsigned long long)(t - te));
     atomicAdd(&d.tt_n[e], 1);
   }
+}
+
+// Barrier of all blocks of a cooperative launch, bounded by `limit` SM cycles (false: it ran
+// out here or in another block; kErrTimeout is set).
+__device__ __forceinline__ bool grid_barrier(GridSync* gs, int* err, long long limit) {
+  __shared__ int s_ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    volatile unsigned* vgen = &gs->gen;
+    volatile int* verr = err;
+    const unsigned g = *vgen;
+    __threadfence();
+    const unsigned arrived = atomicAdd(&gs->count, 1u);
+    if (arrived == gridDim.x - 1) {
+      gs->count = 0;
+      __threadfence();
+      atomicAdd(&gs->gen, 1u);
+    } else {
+      const long long t0 = clock64();
+      while (*vgen == g) {
+        if ((*verr & kErrTimeout) || clock64() - t0 > limit) {
+          atomicOr(err, kErrTimeout);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    __threadfence();
+    if (*verr & kErrTimeout) ok = 0;
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
 }
 
 // ------------------------------------------------------------------ departures
