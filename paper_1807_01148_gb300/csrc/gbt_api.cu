@@ -985,8 +985,9 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
   if ((long long)nn * cmax >= 2000000000LL) return fail(h, SIM_EINVAL, "path costs could overflow int32");
   for (int i = 0; i < nt; i++)
     if (h->origin[i] == h->dest[i]) return fail(h, SIM_EINVAL, "trip with origin == destination");
-  // CSR of out-links and in-links (ascending link id), trips by origin
-  std::vector<int32_t> os(nn + 1, 0), ol(nl), is(nn + 1, 0), il(nl), ts(nn + 1, 0), tl(nt > 0 ? nt : 1);
+  // out-links and in-links (ascending link id) with their costs by node, trips by origin
+  std::vector<int32_t> os(nn + 1, 0), is(nn + 1, 0), il(nl), ts(nn + 1, 0), tl(nt > 0 ? nt : 1);
+  std::vector<int2> oe(nl), ie(nl);
   for (int e = 0; e < nl; e++) {
     os[h->lfrom[e] + 1]++;
     is[h->lto[e] + 1]++;
@@ -1001,8 +1002,10 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
   {
     std::vector<int32_t> fo(os.begin(), os.end() - 1), fi(is.begin(), is.end() - 1), ft(ts.begin(), ts.end() - 1);
     for (int e = 0; e < nl; e++) {
-      ol[fo[h->lfrom[e]]++] = e;
-      il[fi[h->lto[e]]++] = e;
+      oe[fo[h->lfrom[e]]++] = make_int2(h->lto[e], cost[e]);
+      const int q = fi[h->lto[e]]++;
+      ie[q] = make_int2(h->lfrom[e], cost[e]);
+      il[q] = e;
     }
     for (int i = 0; i < nt; i++)
       if (!sel || (*sel)[i]) tl[ft[h->origin[i]]++] = i;
@@ -1018,9 +1021,10 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
   // link costs at most 1e6.
   const int delta = (int)std::max<long long>(1, 8 * csum / std::max(1, nl));
 
-  // four trees in flight per SM (one per 256-thread block): a tree's rounds are short and
-  // synchronous, so more trees hide more of their latency
-  const int n_cta = std::max(1, std::min<int>((int)origins.size(), h->sm_count * 4));
+  // eight trees in flight per SM (one per 256-thread block): a tree's rounds are short and
+  // synchronous, so more trees hide more of their latency (12,000 metro trees 49 ms with
+  // four, 43 with eight); four where the memory cap does not leave room for more
+  int n_cta = std::max(1, std::min<int>((int)origins.size(), h->sm_count * 8));
   std::vector<void*> tmp;
   auto talloc = [&](auto** p, size_t n) -> int {
     int rc = dalloc(h, p, n);
@@ -1034,57 +1038,68 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
 
   RouteDev R{};
   int rc = SIM_OK;
-  int32_t *dos, *dol, *dis, *dil, *dlt, *dcost, *dorig, *dts, *dtl, *ddest;
-  if ((rc = talloc(&dos, os.size())) || (rc = talloc(&dol, ol.size())) || (rc = talloc(&dis, is.size())) ||
-      (rc = talloc(&dil, il.size())) || (rc = talloc(&dlt, (size_t)nl)) || (rc = talloc(&dcost, (size_t)nl)) ||
+  int32_t *dos, *dis, *dil, *dorig, *dts, *dtl, *ddest;
+  int2 *doe, *die;
+  if ((rc = talloc(&dos, os.size())) || (rc = talloc(&doe, oe.size())) || (rc = talloc(&dis, is.size())) ||
+      (rc = talloc(&die, ie.size())) || (rc = talloc(&dil, il.size())) ||
       (rc = talloc(&dorig, origins.size() + 1)) || (rc = talloc(&dts, ts.size())) ||
       (rc = talloc(&dtl, tl.size())) || (rc = talloc(&ddest, (size_t)std::max(1, nt)))) {
     cleanup();
     return rc;
   }
   cudaMemcpy(dos, os.data(), os.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dol, ol.data(), ol.size() * 4, cudaMemcpyHostToDevice);
+  cudaMemcpy(doe, oe.data(), oe.size() * 8, cudaMemcpyHostToDevice);
   cudaMemcpy(dis, is.data(), is.size() * 4, cudaMemcpyHostToDevice);
+  cudaMemcpy(die, ie.data(), ie.size() * 8, cudaMemcpyHostToDevice);
   cudaMemcpy(dil, il.data(), il.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dlt, h->lto.data(), (size_t)nl * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dcost, cost.data(), (size_t)nl * 4, cudaMemcpyHostToDevice);
   if (!origins.empty()) cudaMemcpy(dorig, origins.data(), origins.size() * 4, cudaMemcpyHostToDevice);
   cudaMemcpy(dts, ts.data(), ts.size() * 4, cudaMemcpyHostToDevice);
   cudaMemcpy(dtl, tl.data(), tl.size() * 4, cudaMemcpyHostToDevice);
   if (nt) cudaMemcpy(ddest, h->dest.data(), (size_t)nt * 4, cudaMemcpyHostToDevice);
-  const size_t per = (size_t)n_cta * (size_t)nn;
-  unsigned long long* ddist;
-  int32_t *qf, *ff, *qa, *qb, *fa, *fb, *cround;
+  RouteNode* dnode;
+  int32_t *qa, *qb, *fa, *fb, *cround;
   unsigned* cep;
   int* work;
-  if ((rc = talloc(&ddist, per)) || (rc = talloc(&qf, per)) || (rc = talloc(&ff, per)) || (rc = talloc(&qa, per)) ||
-      (rc = talloc(&qb, per)) || (rc = talloc(&fa, per)) || (rc = talloc(&fb, per)) ||
-      (rc = talloc(&cround, (size_t)n_cta)) || (rc = talloc(&cep, (size_t)n_cta)) || (rc = talloc(&work, 1))) {
-    cleanup();
-    return rc;
+  const size_t n_tables = tmp.size();
+  for (;;) {
+    const size_t per = (size_t)n_cta * (size_t)nn;
+    rc = SIM_OK;
+    if ((rc = talloc(&dnode, per)) || (rc = talloc(&qa, per)) || (rc = talloc(&qb, per)) || (rc = talloc(&fa, per)) ||
+        (rc = talloc(&fb, per)) || (rc = talloc(&cround, (size_t)n_cta)) || (rc = talloc(&cep, (size_t)n_cta)) ||
+        (rc = talloc(&work, 1))) {
+      if (rc == SIM_ENOMEM && n_cta > h->sm_count * 4) {
+        cudaGetLastError();
+        n_cta = h->sm_count * 4;
+        while (tmp.size() > n_tables) {
+          dfree(h, tmp.back());
+          tmp.pop_back();
+        }
+        continue;
+      }
+      cleanup();
+      return rc;
+    }
+    break;
   }
-  cudaMemset(ddist, 0xFF, per * 8);
-  cudaMemset(qf, 0, per * 4);
-  cudaMemset(ff, 0, per * 4);
+  const size_t per = (size_t)n_cta * (size_t)nn;
+  // distances beyond every epoch; the queue tags of -1 equal no round and no epoch (both
+  // count up from 1)
+  cudaMemset(dnode, 0xFF, per * sizeof(RouteNode));
   cudaMemset(cround, 0, (size_t)n_cta * 4);
   cudaMemset(cep, 0, (size_t)n_cta * 4);
   R.nn = nn;
   R.nl = nl;
   R.out_start = dos;
-  R.out_link = dol;
+  R.out_edge = doe;
   R.in_start = dis;
+  R.in_edge = die;
   R.in_link = dil;
-  R.lfrom = h->d.lfrom;
-  R.lto = dlt;
-  R.cost = dcost;
   R.origins = dorig;
   R.n_origins = (int)origins.size();
   R.otrip_start = dts;
   R.otrip_list = dtl;
   R.dest = ddest;
-  R.dist = ddist;
-  R.qflag = qf;
-  R.fflag = ff;
+  R.node = dnode;
   R.qa = qa;
   R.qb = qb;
   R.fa = fa;

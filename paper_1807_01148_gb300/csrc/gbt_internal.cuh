@@ -298,25 +298,32 @@ struct Dev {
   long long wait_limit;            // SM cycles a staging wait of the chunk kernel may take
 };
 
+// Search state of a node in one tree: tentative distance under the tree's epoch tag, round
+// that last queued the node, epoch that last put it on the far pile.  One 16-byte record, so
+// that a relaxation touches one sector.
+struct __align__(16) RouteNode {
+  unsigned long long key;
+  int32_t q, f;
+};
+
 // Trip-planning work description (one shortest-path tree per distinct origin).
 struct RouteDev {
   int nn, nl;
   const int32_t* out_start;
-  const int32_t* out_link;
-  const int32_t* in_start;
-  const int32_t* in_link;
-  const int32_t* lfrom;
-  const int32_t* lto;
+  const int2* out_edge;         // by tail node: (head, cost); null: the three arrays below
+  const int32_t* out_link;      // by tail node: link ids
+  const int32_t* lto;           // per link
   const int32_t* cost;
+  const int32_t* in_start;
+  const int2* in_edge;          // by head node, ascending link id: (tail, cost)
+  const int32_t* in_link;       // their link ids
   const int32_t* origins;
   int n_origins;
   const int32_t* otrip_start;   // per node: trips with this origin
   const int32_t* otrip_list;
   const int32_t* dest;
-  unsigned long long* dist;     // [n_cta][nn]
-  int32_t* qflag;
-  int32_t* fflag;
-  int32_t* qa;
+  RouteNode* node;              // [n_cta][nn]
+  int32_t* qa;                  // [n_cta][nn] each
   int32_t* qb;
   int32_t* fa;
   int32_t* fb;

@@ -11,7 +11,7 @@
 //
 // The search itself is the same near-far kernel sim_route runs per origin; its
 // distance and flag words carry an epoch / round tag, so the array never needs
-// clearing between calls: the distance words are filled with all-ones once, when
+// clearing between calls: the node records are filled with all-ones once, when
 // a device is first used, and only the small per-call block (work counter, error
 // word, cost sums) is cleared at the start of every call.
 #include <algorithm>
@@ -46,17 +46,15 @@ struct StaticCall {
 
 constexpr size_t kOffPersist = 0;
 constexpr size_t kOffCall = 256;
-constexpr size_t kOffDist = 1024;                        // 8 B x kN, epoch-tagged distances
-constexpr size_t kOffQflag = kOffDist + 8 * kN;          // 4 B x kN each below
-constexpr size_t kOffFflag = kOffQflag + 4 * kN;
-constexpr size_t kOffQa = kOffFflag + 4 * kN;
+constexpr size_t kOffNode = 1024;                        // kN node records (epoch-tagged distances, queue tags)
+constexpr size_t kOffQa = kOffNode + sizeof(RouteNode) * kN;   // 4 B x kN each below
 constexpr size_t kOffQb = kOffQa + 4 * kN;
 constexpr size_t kOffFa = kOffQb + 4 * kN;
 constexpr size_t kOffFb = kOffFa + 4 * kN;
 constexpr size_t kOffZeros = kOffFb + 4 * kN;            // kN + 1 zeros: "no trips at any node"
 constexpr size_t kStaticBytes = kOffZeros + 4 * (kN + 1) + 256;
 static_assert(sizeof(StaticPersist) <= kOffCall - kOffPersist, "persist block too large");
-static_assert(sizeof(StaticCall) <= kOffDist - kOffCall, "call block too large");
+static_assert(sizeof(StaticCall) <= kOffNode - kOffCall, "call block too large");
 
 // The working memory.  Zero at module load; only this file's host code takes its
 // address, through cudaGetSymbolAddress.
@@ -70,7 +68,7 @@ std::mutex g_scratch_mu;
 // The search tags distance words with an epoch and queue flags with a round number,
 // both counted up for the life of the array.  Before either could wrap around (which
 // would make stale words look current), the array is put back to its first-use state:
-// distance words all-ones, flags zero, counters zero.  Both are read back after every
+// node records all-ones, counters zero.  Both are read back after every
 // call; the reset happens once either passes this bound (about a billion calls or
 // rounds), far below the 2^31 where the comparisons would break.
 constexpr unsigned kCounterResetAt = 1u << 30;
@@ -109,10 +107,10 @@ __global__ void k_static_begin(StaticCall* call, int origin) {
 // The search kernel takes a new epoch each time it asks for work, including the last
 // request that finds none, so the tree of this call carries the epoch before the
 // counter's final value.
-__global__ void k_static_dist_out(int n, const unsigned long long* dist, const StaticPersist* ps, int32_t* out) {
+__global__ void k_static_dist_out(int n, const RouteNode* node, const StaticPersist* ps, int32_t* out) {
   const unsigned hi = 0xFFFFFFFFu - (ps->cta_epoch - 1u);
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-    const unsigned long long k = dist[v];
+    const unsigned long long k = node[v].key;
     out[v] = (unsigned)(k >> 32) == hi ? (int32_t)(unsigned)k : INT32_MAX;
   }
 }
@@ -125,9 +123,10 @@ int scratch_address(unsigned char** out) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_sssp_scratch) != cudaSuccess || !p) return SIM_ECUDA;
     // A distance word compares as newer the smaller it is; the array starts at zero,
-    // which would beat every real distance, so it is filled with all-ones once.
+    // which would beat every real distance, so the node records are filled with all-ones once
+    // (queue tags of -1 equal no round and no epoch).
     unsigned char* b = static_cast<unsigned char*>(p);
-    if (cudaMemset(b + kOffDist, 0xFF, 8 * kN) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
+    if (cudaMemset(b + kOffNode, 0xFF, sizeof(RouteNode) * kN) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
       return SIM_ECUDA;
     g_scratch_addr[dev] = b;
   }
@@ -173,9 +172,7 @@ extern "C" int sim_sssp_static(int32_t n_nodes, int32_t n_links, const int32_t* 
   R.origins = &call->origin;
   R.n_origins = 1;
   R.otrip_start = reinterpret_cast<const int32_t*>(base + kOffZeros);
-  R.dist = reinterpret_cast<unsigned long long*>(base + kOffDist);
-  R.qflag = reinterpret_cast<int32_t*>(base + kOffQflag);
-  R.fflag = reinterpret_cast<int32_t*>(base + kOffFflag);
+  R.node = reinterpret_cast<RouteNode*>(base + kOffNode);
   R.qa = reinterpret_cast<int32_t*>(base + kOffQa);
   R.qb = reinterpret_cast<int32_t*>(base + kOffQb);
   R.fa = reinterpret_cast<int32_t*>(base + kOffFa);
@@ -189,15 +186,14 @@ extern "C" int sim_sssp_static(int32_t n_nodes, int32_t n_links, const int32_t* 
   k_static_begin<<<1, 1, 0, s>>>(call, origin);
   launch_route(R, 1, s);
   const int g2 = (n_nodes + 255) / 256;
-  k_static_dist_out<<<g2 < 1024 ? g2 : 1024, 256, 0, s>>>(n_nodes, R.dist, ps, dist_out);
+  k_static_dist_out<<<g2 < 1024 ? g2 : 1024, 256, 0, s>>>(n_nodes, R.node, ps, dist_out);
   if (cudaGetLastError() != cudaSuccess) return SIM_ECUDA;
   StaticPersist hp;
   if (cudaMemcpyAsync(&hp, ps, sizeof(hp), cudaMemcpyDeviceToHost, s) != cudaSuccess) return SIM_ECUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return SIM_ECUDA;
   if (hp.cta_epoch >= kCounterResetAt || (unsigned)hp.cta_round >= kCounterResetAt) {
     // back to the first-use state (see kCounterResetAt); this call's output is complete
-    if (cudaMemsetAsync(base + kOffDist, 0xFF, 8 * kN, s) != cudaSuccess ||
-        cudaMemsetAsync(base + kOffQflag, 0, 8 * kN, s) != cudaSuccess ||   // queue and far flags
+    if (cudaMemsetAsync(base + kOffNode, 0xFF, sizeof(RouteNode) * kN, s) != cudaSuccess ||
         cudaMemsetAsync(ps, 0, sizeof(StaticPersist), s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
       return SIM_ECUDA;
   }
