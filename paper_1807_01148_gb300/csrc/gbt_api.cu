@@ -18,7 +18,7 @@ void launch_step(const Dev& d, int grid, bool has_stop, cudaStream_t s);
 void launch_occupancy(const Dev& d, int grid, cudaStream_t s);
 void launch_count(const Dev& d, int grid, cudaStream_t s);
 int scan_blocks(int n_lanes);
-void launch_state_out(const Dev& d, int grid, cudaStream_t s, bool seg, uint8_t* status, int32_t* link, int32_t* lane,
+void launch_state_out(const SegDev& d, int grid, cudaStream_t s, bool seg, uint8_t* status, int32_t* link, int32_t* lane,
                       int32_t* cursor, float* x, float* v, int32_t* ins, int32_t* arr, int8_t* dec);
 void launch_state_in(const Dev& d, int grid, cudaStream_t s, const uint8_t* status, const int32_t* link,
                      const int32_t* lane, const int32_t* cursor, const float* x, const float* v);
@@ -30,7 +30,8 @@ cudaError_t launch_steps_timed(const Dev& d, int grid, bool has_stop, cudaStream
 void launch_observe(const Dev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out);
 void launch_tape_begin(const Dev& d, cudaStream_t s);
 void launch_adj_step(const Dev& d, int grid, cudaStream_t s, const TapeRec* slab, const double* lx,
-                     const double* lv, const double* res, double* nx, double* nv, double* grad, int n_class);
+                     const double* lv, const double* res, double* nx, double* nv, double* zx, double* zv, double* grad,
+                     int n_class);
 void launch_first_links(const int32_t* roff, const int32_t* routes, int n, int32_t* out, cudaStream_t s);
 void launch_measured_costs(const Dev& d, const int32_t* prev, int32_t* out, cudaStream_t s);
 void launch_fw_t0(const float* len, const float* spd, double* t0, int n, cudaStream_t s);
@@ -51,16 +52,16 @@ void launch_fw_final_time(const double* t0, const double* x, const double* cap, 
                           int n, cudaStream_t s);
 void launch_compact_routes(const int32_t* roff, const int32_t* rlen, const int32_t* src, const int32_t* new_off,
                            int32_t* dst, int n, cudaStream_t s);
-void launch_seg_step(const Dev& d, int grid, cudaStream_t s);
-cudaError_t launch_seg_steps_timed(const Dev& d, int grid, cudaStream_t s, int n, float* ms);
-cudaError_t launch_seg_import(const Dev& d, int grid, cudaStream_t s);
-cudaError_t launch_seg_export(const Dev& d, int grid, cudaStream_t s);
-void launch_seg_lane_stat(const Dev& d, int grid, cudaStream_t s);
-void launch_seg_observe(const Dev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out);
-cudaError_t launch_seg_persistent(const Dev& d, GridSync* gs, int blocks, int threads, int n_steps, long long limit,
+void launch_seg_step(const SegDev& d, int grid, cudaStream_t s);
+cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, int n, float* ms);
+cudaError_t launch_seg_import(const SegDev& d, int grid, cudaStream_t s);
+cudaError_t launch_seg_export(const SegDev& d, int grid, cudaStream_t s);
+void launch_seg_lane_stat(const SegDev& d, int grid, cudaStream_t s);
+void launch_seg_observe(const SegDev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out);
+cudaError_t launch_seg_persistent(const SegDev& d, GridSync* gs, int blocks, int threads, int n_steps, long long limit,
                                   cudaStream_t s);
 bool seg_persistent_fits(int threads, int per_sm);
-void seg_grids(Dev& d, int sm_count);
+void seg_grids(SegDev& d, int sm_count);
 void seg_capacities(int n_links, const float* len, const uint8_t* lanes, int n_trips, float vlen_min,
                     const int32_t* now, std::vector<int32_t>& cap);
 int seg_slots(int n_links, const uint8_t* lanes, std::vector<int32_t>& lslot);
@@ -85,6 +86,21 @@ struct NvtxRange {
   ~NvtxRange() { nvtxRangePop(); }
   NvtxRange(const NvtxRange&) = delete;
   NvtxRange& operator=(const NvtxRange&) = delete;
+};
+
+// Steps captured into one graph where several follow each other: what a graph launch costs
+// between two steps (about 2 us) is then paid once per kUnroll steps.
+constexpr int kUnroll = 8;
+struct StepGraph {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  size_t nodes = 0;
+  void drop() {
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
+    exec = nullptr;
+    graph = nullptr;
+  }
 };
 
 struct HostMirror {
@@ -113,7 +129,6 @@ struct sim_handle {
   std::vector<double> lane_m;   // lanes x length per link (chunk_split_needed)
   double max_len = 0.0;         // longest link (rank_long_needed)
   long long launches = 0;    // kernel launches made by sim_step (sim_launch_count)
-  size_t graph_nodes = 0, graph_samp_nodes = 0;   // kernels per step of the step graphs
   // host copies
   std::vector<int32_t> lfrom, lto, depart, origin, dest, node_x, node_y;
   std::vector<float> len, spd;
@@ -124,7 +139,7 @@ struct sim_handle {
   std::vector<void*> allocs;
   std::vector<size_t> alloc_sizes;   // bytes of each entry of allocs
   size_t bytes = 0, max_bytes = 0;   // device bytes held; cap (0: none)
-  Dev d{};
+  SegDev d{};
   int32_t* routes = nullptr;
   unsigned long long route_cap = 0;
   int32_t* q_items = nullptr;
@@ -132,12 +147,11 @@ struct sim_handle {
   int32_t* q_head = nullptr;
   int32_t* qlinks = nullptr;
   bool routed = false;
-  cudaGraphExec_t gexec = nullptr;
-  cudaGraph_t graph = nullptr;
+  // captured steps: one, kUnroll in a row, one with the per-edge sample kernel (launched at
+  // sampling instants only); the taping ones of the adjoint
+  StepGraph step1, step8, samp1, tape1, tape8;
+  int steps_run = 0, tape_steps_run = 0;   // steps made with the present ones
   bool graph_dirty = true;
-  // the step graph with the per-edge sample kernel, launched at sampling instants only
-  cudaGraphExec_t gexec_samp = nullptr;
-  cudaGraph_t graph_samp = nullptr;
   // class parameters (host copies) and the adjoint's tape
   std::vector<float> v0c, Tc, ac, bc, s0c, spd_link;
   std::vector<uint8_t> cls_link;
@@ -145,8 +159,6 @@ struct sim_handle {
   TapeRec* tape = nullptr;
   TapeForm* tform = nullptr;
   int tape_steps = 0;
-  cudaGraphExec_t gexec_tape = nullptr;
-  cudaGraph_t graph_tape = nullptr;
   bool tape_graph_dirty = true;
   // execution configuration of sim_step
   sim_exec exec{SIM_EXEC_GRAPH, 256, 0, 8, 0};
@@ -286,7 +298,7 @@ bool seg_release(sim_handle* h) {
 // Segments and the static tables of the segment form.  now (or null): vehicles per link that
 // must fit.  SIM_ENOMEM leaves nothing allocated.
 int seg_alloc(sim_handle* h, const int32_t* now) {
-  Dev& d = h->d;
+  SegDev& d = h->d;
   const int nl = h->nl;
   float vmin = d.vlen;
   for (float v : h->vty_len) vmin = std::min(vmin, v);
@@ -316,14 +328,15 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
     lnext[e] = LinkNext{(int32_t)hx, (int32_t)hy, lslot[e] << 3 | (h->lanes[e] - 1), 0};
   }
   // in-links of every node in ascending id, and every link's tail among them
-  std::vector<int32_t> start(h->nn + 1, 0), nin((size_t)nl), tail((size_t)nl);
+  std::vector<int32_t> start(h->nn + 1, 0), nin((size_t)nl), tail(ns, 0);
   for (int e = 0; e < nl; e++) start[h->lto[e] + 1]++;
   for (int v = 0; v < h->nn; v++) start[v + 1] += start[v];
   {
     std::vector<int32_t> fill(start.begin(), start.end() - 1);
     for (int e = 0; e < nl; e++) nin[fill[h->lto[e]]++] = lslot[e];
   }
-  for (int e = 0; e < nl; e++) tail[e] = start[h->lfrom[e]];
+  for (int e = 0; e < nl; e++)
+    for (int l = 0; l < h->lanes[e]; l++) tail[(size_t)lslot[e] + l] = start[h->lfrom[e]];
   h->seg_building = true;
   int rc = SIM_OK;
   auto get = [&](auto** p, size_t n, const void* src = nullptr) {
@@ -347,7 +360,7 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   get(&d.cr2, ns);
   get(&d.lnext, (size_t)nl, lnext.data());
   get(&d.lslot, (size_t)nl, lslot.data());
-  get(&d.tail_in, (size_t)nl, tail.data());
+  get(&d.stail, ns, tail.data());
   get(&d.nin_slot, (size_t)nl, nin.data());
   get(&d.qnext, ns);
   get(&d.big_links, (size_t)std::max(1, n_big));
@@ -408,6 +421,12 @@ int seg_from_sorted(sim_handle* h) {
   CK(cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream));
   launch_count(h->d, h->grid, h->stream);
   return SIM_OK;
+}
+
+// Route progress of the present state, in either form (see k_observe).
+void observe(sim_handle* h, const double* target, double* res, double* p_out) {
+  if (h->seg) launch_seg_observe(h->d, h->grid, h->stream, target, res, p_out);
+  else launch_observe(h->d, h->grid, h->stream, target, res, p_out);
 }
 
 // The form the next steps run in.
@@ -1348,32 +1367,57 @@ int sim_read_routes(sim_handle* h, int32_t* offsets, int32_t* links) {
 
 namespace {
 
-// The step graph of the present form (and, with edge samples on, the one of the sampling
-// instants).
-int build_step_graph(sim_handle* h) {
-  if (!h->graph_dirty && h->graph_seg == h->seg) return SIM_OK;
-  if (h->gexec) cudaGraphExecDestroy(h->gexec);
-  if (h->graph) cudaGraphDestroy(h->graph);
-  if (h->gexec_samp) cudaGraphExecDestroy(h->gexec_samp);
-  if (h->graph_samp) cudaGraphDestroy(h->graph_samp);
-  h->gexec = h->gexec_samp = nullptr;
-  h->graph = h->graph_samp = nullptr;
-  auto capture = [&](const Dev& d, cudaGraph_t* g, cudaGraphExec_t* x, size_t* nodes) -> int {
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+// Capture n steps in the present form into G, if it is not there already.
+int capture_steps(sim_handle* h, StepGraph& G, const SegDev& d, int n) {
+  if (G.exec) return SIM_OK;
+  CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  for (int k = 0; k < n; k++) {
     if (h->seg) launch_seg_step(d, h->grid, h->cap_stream);
     else launch_step(d, h->grid, h->has_stop, h->cap_stream);
-    CK(cudaStreamEndCapture(h->cap_stream, g));
-    CK(cudaGraphInstantiate(x, *g, 0));
-    CK(cudaGraphGetNodes(*g, nullptr, nodes));
-    return SIM_OK;
-  };
-  Dev dn = h->d;
-  dn.acc_u = nullptr;   // steps between sampling instants skip the sample kernel
-  if (int rc = capture(dn, &h->graph, &h->gexec, &h->graph_nodes)) return rc;
-  if (h->d.acc_u)
-    if (int rc = capture(h->d, &h->graph_samp, &h->gexec_samp, &h->graph_samp_nodes)) return rc;
-  h->graph_dirty = false;
-  h->graph_seg = h->seg;
+  }
+  cudaError_t e = cudaStreamEndCapture(h->cap_stream, &G.graph);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(&G.exec, G.graph, 0);
+  if (e == cudaSuccess) e = cudaGraphGetNodes(G.graph, nullptr, &G.nodes);
+  if (e != cudaSuccess) {
+    G.drop();
+    return cuda_fail(h, e, "step graph");
+  }
+  return SIM_OK;
+}
+
+// n steps as graphs: kUnroll at a time, then one by one.  Without tape: the plain steps of
+// sim_step (no edge sample); with it: the adjoint's taping steps.
+int enqueue_graph_steps(sim_handle* h, int n, bool tape, bool count) {
+  bool& dirty = tape ? h->tape_graph_dirty : h->graph_dirty;
+  bool& form = tape ? h->tape_graph_seg : h->graph_seg;
+  int& steps = tape ? h->tape_steps_run : h->steps_run;
+  StepGraph &g1 = tape ? h->tape1 : h->step1, &g8 = tape ? h->tape8 : h->step8;
+  if (dirty || form != h->seg) {
+    g1.drop();
+    g8.drop();
+    if (!tape) h->samp1.drop();
+    steps = 0;
+    dirty = false;
+    form = h->seg;
+  }
+  if (n <= 0) return SIM_OK;
+  SegDev d = h->d;
+  d.acc_u = nullptr;   // steps between sampling instants skip the sample kernel
+  if (tape) {
+    d.tape = h->tape;
+    d.tform = h->tform;
+  }
+  for (int k = 0; k < n;) {
+    // (the longer graph only once enough steps were made to pay for its capture)
+    const bool many = n - k >= kUnroll && (g8.exec || n >= 8 * kUnroll || steps >= 8 * kUnroll);
+    const int m = many ? kUnroll : 1;
+    StepGraph& G = m > 1 ? g8 : g1;
+    if (int rc = capture_steps(h, G, d, m)) return rc;
+    CK(cudaGraphLaunch(G.exec, h->stream));
+    if (count) h->launches += (long long)G.nodes;
+    k += m;
+    steps = std::min(steps + m, 1 << 20);
+  }
   return SIM_OK;
 }
 
@@ -1422,18 +1466,26 @@ int enqueue_steps(sim_handle* h, long long t0, int n_steps) {
     h->launches += 1;
     return SIM_OK;
   }
-  if (int rc = build_step_graph(h)) return rc;
   const long long every = h->d.acc_u ? h->d.samp_every : 0;
-  for (int s = 0; s < n_steps; s++) {
-    const bool samp = every > 0 && (t0 + s) % every == 0;
-    CK(cudaGraphLaunch(samp ? h->gexec_samp : h->gexec, h->stream));
-    h->launches += (long long)(samp ? h->graph_samp_nodes : h->graph_nodes);
+  for (int s = 0; s < n_steps;) {
+    if (every > 0 && (t0 + s) % every == 0) {   // a sampling instant
+      if (int rc = enqueue_graph_steps(h, 0, false, true)) return rc;
+      if (int rc = capture_steps(h, h->samp1, h->d, 1)) return rc;
+      CK(cudaGraphLaunch(h->samp1.exec, h->stream));
+      h->launches += (long long)h->samp1.nodes;
+      s++;
+      continue;
+    }
+    int n = n_steps - s;
+    if (every > 0) n = (int)std::min<long long>(n, every - (t0 + s) % every);
+    if (int rc = enqueue_graph_steps(h, n, false, true)) return rc;
+    s += n;
   }
   return SIM_OK;
 }
 
-// After steps that stopped before step `upto` because a segment was full (the step they
-// stopped at has not begun): back to the sorted form, larger segments or none.
+// After steps that stopped because a segment was full (the step they stopped at has not
+// begun): back to the sorted form, larger segments or none.
 int seg_regrow(sim_handle* h, int grow) {
   if (int rc = seg_to_sorted(h)) return rc;
   if (grow != 2) return SIM_OK;   // seg_from_sorted lays it out again
@@ -1785,7 +1837,7 @@ int sim_observe(sim_handle* h, int32_t n_steps, int32_t obs_every, double* progr
   if (rc) return rc;
   for (int k = 0; k < nobs; k++) {
     if ((rc = sim_step(h, obs_every))) break;
-    (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, nullptr, nullptr, dp);
+    observe(h, nullptr, nullptr, dp);
     cudaError_t e = cudaMemcpyAsync(progress + (size_t)k * nt, dp, nt * 8, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
@@ -1821,7 +1873,7 @@ int sim_loss(sim_handle* h, const sim_loss_spec* spec, double* loss_out) {
   if (e != cudaSuccess) rc = cuda_fail(h, e, "loss");
   for (int k = 0; k < nobs && rc == SIM_OK; k++) {
     if ((rc = sim_step(h, every))) break;
-    (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, tgt + (size_t)k * nt, res, nullptr);
+    observe(h, tgt + (size_t)k * nt, res, nullptr);
   }
   if (rc == SIM_OK) {
     e = cudaMemcpyAsync(loss_out, &h->d.ctl->loss, 8, cudaMemcpyDeviceToHost, h->stream);
@@ -1853,7 +1905,7 @@ CkptLayout ckpt_layout(const sim_handle* h) {
 
 cudaError_t ckpt_copy(sim_handle* h, unsigned char* buf, bool save) {
   const CkptLayout L = ckpt_layout(h);
-  Dev& d = h->d;
+  SegDev& d = h->d;
   // checkpoints hold the sorted form
   if (save && h->seg) {
     cudaError_t e = launch_seg_export(d, h->grid, h->stream);
@@ -1938,44 +1990,22 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
     release();
     return rc;
   }
-  auto graphs = [&]() -> int {
-    if (int r = build_step_graph(h)) return r;
-    if (!h->tape_graph_dirty && h->tape_graph_seg == h->seg) return SIM_OK;
-    if (h->gexec_tape) cudaGraphExecDestroy(h->gexec_tape);
-    if (h->graph_tape) cudaGraphDestroy(h->graph_tape);
-    h->gexec_tape = nullptr;
-    h->graph_tape = nullptr;
-    Dev dt = h->d;
-    dt.tape = h->tape;
-    dt.tform = h->tform;
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    if (h->seg) launch_seg_step(dt, h->grid, h->cap_stream);
-    else launch_step(dt, h->grid, h->has_stop, h->cap_stream);
-    CK(cudaStreamEndCapture(h->cap_stream, &h->graph_tape));
-    CK(cudaGraphInstantiate(&h->gexec_tape, h->graph_tape, 0));
-    h->tape_graph_dirty = false;
-    h->tape_graph_seg = h->seg;
-    return SIM_OK;
-  };
-  if ((rc = graphs())) {
-    release();
-    return rc;
-  }
   const int ng = h->ncls * 5;
   cudaError_t e = cudaMemcpyAsync(tgt, spec->target, (size_t)nobs * nt * 8, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, (size_t)ng * 8, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->loss, 0, 8, h->stream);
   // ---- forward: checkpoint every `seg` steps, observe every `every` steps
   auto forward = [&]() {
-    for (int sg = 0; sg < nseg && e == cudaSuccess; sg++) {
+    for (int sg = 0; sg < nseg && e == cudaSuccess && rc == SIM_OK; sg++) {
       e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, true);
       const int j1 = std::min(n_steps, (sg + 1) * seg);
-      for (int j = sg * seg; j < j1 && e == cudaSuccess; j++) {
-        e = cudaGraphLaunch(h->gexec, h->stream);
-        if ((j + 1) % every == 0) {
-          const int k = (j + 1) / every - 1;
-          (h->seg ? launch_seg_observe : launch_observe)(h->d, h->grid, h->stream, tgt + (size_t)k * nt,
-                                                         res + (size_t)k * nt, nullptr);
+      for (int j = sg * seg; j < j1 && e == cudaSuccess && rc == SIM_OK;) {
+        const int n = std::min(j1 - j, every - j % every);   // up to the next observation
+        rc = enqueue_graph_steps(h, n, false, false);
+        j += n;
+        if (j % every == 0) {
+          const int k = j / every - 1;
+          observe(h, tgt + (size_t)k * nt, res + (size_t)k * nt, nullptr);
         }
       }
     }
@@ -1990,31 +2020,36 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
       if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->loss, 0, 8, h->stream);
       h->seg_off = true;
-      if ((rc = graphs())) {
-        release();
-        return rc;
-      }
       forward();
     }
   }
   const bool replay_seg = h->seg;
   if (e == cudaSuccess) e = ckpt_copy(h, ck + (size_t)nseg * CL.bytes, true);   // end state
   // ---- reverse: per segment, replay it with the tape, then sweep it backwards
+  // adjoints after and before a step, and a pair that the step clears for the one before it:
+  // the targets' memory, idle by now (one observation: no room there, cleared by a memset)
   double *lx = lam, *lv = lam + nt, *nx = lam + 2 * nt, *nv = lam + 3 * nt;
-  if (e == cudaSuccess) e = cudaMemsetAsync(lam, 0, 2 * nt * 8, h->stream);
-  for (int sg = nseg - 1; sg >= 0 && e == cudaSuccess; sg--) {
+  double *zx = nobs >= 2 ? tgt : nullptr, *zv = nobs >= 2 ? tgt + nt : nullptr;
+  if (e == cudaSuccess) e = cudaMemsetAsync(lam, 0, 4 * nt * 8, h->stream);
+  for (int sg = nseg - 1; sg >= 0 && e == cudaSuccess && rc == SIM_OK; sg--) {
     const int j0 = sg * seg, j1 = std::min(n_steps, (sg + 1) * seg);
     e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, false);
     if (e == cudaSuccess && replay_seg) e = launch_seg_import(h->d, h->grid, h->stream);   // fits: the forward pass did
     if (e == cudaSuccess) e = cudaMemsetAsync(h->tape, 0, (size_t)seg * nt * sizeof(TapeRec), h->stream);
     launch_tape_begin(h->d, h->stream);
-    for (int j = j0; j < j1 && e == cudaSuccess; j++) e = cudaGraphLaunch(h->gexec_tape, h->stream);
+    h->seg = replay_seg;
+    if (e == cudaSuccess && rc == SIM_OK) rc = enqueue_graph_steps(h, j1 - j0, true, false);
     for (int j = j1 - 1; j >= j0 && e == cudaSuccess; j--) {
-      e = cudaMemsetAsync(nx, 0, 2 * nt * 8, h->stream);
+      if (!zx) e = cudaMemsetAsync(nx, 0, 2 * nt * 8, h->stream);
       const double* r = ((j + 1) % every == 0) ? res + (size_t)((j + 1) / every - 1) * nt : nullptr;
-      launch_adj_step(dtape, h->grid, h->stream, h->tape + (size_t)(j - j0) * nt, lx, lv, r, nx, nv, grad, h->ncls);
-      std::swap(lx, nx);
-      std::swap(lv, nv);
+      launch_adj_step(dtape, h->grid, h->stream, h->tape + (size_t)(j - j0) * nt, lx, lv, r, nx, nv, zx, zv, grad, h->ncls);
+      double *ox = lx, *ov = lv;
+      lx = nx;
+      lv = nv;
+      nx = zx ? zx : ox;
+      nv = zx ? zv : ov;
+      zv = zx ? ov : nullptr;
+      zx = zx ? ox : nullptr;
     }
   }
   if (e == cudaSuccess) e = ckpt_copy(h, ck + (size_t)nseg * CL.bytes, false);
@@ -2022,6 +2057,7 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
   if (e == cudaSuccess) e = cudaMemcpyAsync(loss_out, &h->d.ctl->loss, 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   release();
+  if (rc) return rc;
   if (e != cudaSuccess) return cuda_fail(h, e, "adjoint");
   return check_device(h);
 }
@@ -2458,12 +2494,7 @@ const char* sim_last_error(const sim_handle* h) { return h ? h->err.c_str() : g_
 
 void sim_destroy(sim_handle* h) {
   if (!h) return;
-  if (h->gexec_samp) cudaGraphExecDestroy(h->gexec_samp);
-  if (h->graph_samp) cudaGraphDestroy(h->graph_samp);
-  if (h->gexec) cudaGraphExecDestroy(h->gexec);
-  if (h->graph) cudaGraphDestroy(h->graph);
-  if (h->gexec_tape) cudaGraphExecDestroy(h->gexec_tape);
-  if (h->graph_tape) cudaGraphDestroy(h->graph_tape);
+  for (StepGraph* g : {&h->step1, &h->step8, &h->samp1, &h->tape1, &h->tape8}) g->drop();
   if (h->pexec) cudaGraphExecDestroy(h->pexec);
   if (h->pgraph) cudaGraphDestroy(h->pgraph);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);

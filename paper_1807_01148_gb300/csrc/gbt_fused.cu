@@ -221,6 +221,7 @@ __device__ __forceinline__ void ph_front(const Dev& d, bool split) {
 template <bool TYPES>
 __global__ void __launch_bounds__(256) k_front(Dev d) {
   griddep_wait();
+  griddep_next_small(d);
   if (step_timed_out(d)) return;
   ph_front<TYPES>(d, d.chunk_split != 0);
 }
@@ -667,6 +668,7 @@ __device__ __forceinline__ void ph_chunk(const Dev& d, SMT& S) {
 template <bool OUT, bool TYPES>
 __global__ void __launch_bounds__(kChunkThreads, kChunkMinBlocks) k_chunk(Dev d) {
   griddep_wait();
+  griddep_next_small(d);
   if (step_timed_out(d)) return;
   extern __shared__ __align__(16) unsigned char chunk_smem[];
   ph_chunk<OUT, TYPES, false>(d, *reinterpret_cast<ChunkSmem*>(chunk_smem));
@@ -676,6 +678,7 @@ __global__ void __launch_bounds__(kChunkThreads, kChunkMinBlocks) k_chunk(Dev d)
 template <bool OUT, bool TYPES>
 __global__ void __launch_bounds__(kBigThreads, 2) k_chunk_big(Dev d) {
   griddep_wait();
+  griddep_next_small(d);
   if (step_timed_out(d)) return;
   extern __shared__ __align__(16) unsigned char chunk_smem[];
   ph_chunk<OUT, TYPES, true>(d, *reinterpret_cast<ChunkSmemBig*>(chunk_smem));

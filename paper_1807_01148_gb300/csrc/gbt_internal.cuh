@@ -263,8 +263,19 @@ struct Dev {
   int32_t* q_head;
   const int32_t* q_items;
   Ctl* ctl;
-  // link-segment form of the state (gbt_seg.cuh).  Lanes are numbered by slots there: the
-  // lanes of whole links fill groups of 32 slots, the rest of a group is left empty.
+  int chunk_split;                 // oversized chunks go to the big-chunk launch
+  int rank_long;                   // long lane segments go to k_rank_long
+  int front_grid[2];               // blocks of the lane-front kernel (without / with types)
+  int chunk_grid[8];               // blocks of the chunk kernel (plain, outputs, types, both), then of
+                                   // the big-chunk kernel (same order)
+  long long wait_limit;            // SM cycles a staging wait of the chunk kernel may take
+};
+
+// What the link-segment form of the state adds (gbt_seg.cuh); a type of its own, since every
+// kernel's parameters are copied at its launch (a third more of them cost the sorted form's
+// seven kernels 0.3 to 0.4 us each).  Lanes are numbered by slots: the lanes of whole links
+// fill groups of 32 slots, the rest of a group is left empty.
+struct SegDev : Dev {
   VehRec* rec;                     // link e owns cap records from its segment's start on, in (lane, x, vid) order
   uint32_t* rng;                   // per slot: its vehicles, start relative to the segment | count << 16
   const uint32_t* sinfo;           // per slot: LaneStat::info (control 3: empty slot)
@@ -277,7 +288,7 @@ struct Dev {
   VehRec* cr2;                     // per slot: the bidding front's record after crossing
   const LinkNext* lnext;           // per link
   const int32_t* lslot;            // per link: slot of its lane 0
-  const int32_t* tail_in;          // per link: start of its tail node's in-links in nin_slot
+  const int32_t* stail;            // per slot: start of its link's tail node's in-links in nin_slot
   const int32_t* nin_slot;         // in-links of every node in ascending id: slot of lane 0
   int n_slots;
   int packed;                      // runs are packed by the front phase (else they are parts of a group)
@@ -290,12 +301,6 @@ struct Dev {
   int32_t* late;                   // empty links that a crossing vehicle may enter
   int32_t* claim;                  // per link: t + 1 of the step it was last listed in late
   int seg_front_grid[4], seg_move_grid[6];
-  int chunk_split;                 // oversized chunks go to the big-chunk launch
-  int rank_long;                   // long lane segments go to k_rank_long
-  int front_grid[2];               // blocks of the lane-front kernel (without / with types)
-  int chunk_grid[8];               // blocks of the chunk kernel (plain, outputs, types, both), then of
-                                   // the big-chunk kernel (same order)
-  long long wait_limit;            // SM cycles a staging wait of the chunk kernel may take
 };
 
 // Search state of a node in one tree: tentative distance under the tree's epoch tag, round

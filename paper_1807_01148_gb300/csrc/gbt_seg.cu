@@ -13,17 +13,26 @@
 
 namespace gbt {
 
+// On a network of few groups the next kernel of the step is let in as soon as this one runs:
+// the SMs have room for its blocks, which then wait for this kernel's end with their start-up
+// behind them.  (On a large network they would take the room of running blocks.)
+__device__ __forceinline__ void griddep_next(const SegDev& d) {
+  if (!d.packed) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <bool TYPES, bool TAPE>
-__global__ void __launch_bounds__(256) k_seg_front(Dev d) {
+__global__ void __launch_bounds__(256) k_seg_front(SegDev d) {
   griddep_wait();
+  griddep_next(d);
   if (seg_stopped(d)) return;
   __shared__ SegPack packs[8];
   seg_front<TYPES, TAPE>(d, packs, (int)d.ctl->t);
 }
 
 template <bool OUT, bool TYPES, bool TAPE>
-__global__ void __launch_bounds__(kSegThreads, 4) k_seg_move(Dev d) {
+__global__ void __launch_bounds__(kSegThreads, 4) k_seg_move(SegDev d) {
   griddep_wait();
+  griddep_next(d);
   if (seg_stopped(d)) return;
   extern __shared__ __align__(16) unsigned char seg_smem[];
   seg_move<OUT, TYPES, TAPE>(d, seg_smem, (int)d.ctl->tm);
@@ -31,7 +40,7 @@ __global__ void __launch_bounds__(kSegThreads, 4) k_seg_move(Dev d) {
 
 // Sec. 6.4 per-edge sample of the state at step t (see ph_edge_sample): one thread per link
 // over its segment.
-__device__ __forceinline__ void seg_edge_sample(const Dev& d, long long t) {
+__device__ __forceinline__ void seg_edge_sample(const SegDev& d, long long t) {
   if (t % d.samp_every != 0) return;
   const long long k = t / d.samp_every;
   const long long w = k / d.samp_per;
@@ -64,7 +73,7 @@ __device__ __forceinline__ void seg_edge_sample(const Dev& d, long long t) {
   if (closes && blockIdx.x == 0 && threadIdx.x == 0) d.out_n[w] = (int32_t)(k - from + 1);
 }
 
-__global__ void k_seg_edge_sample(Dev d) {
+__global__ void k_seg_edge_sample(SegDev d) {
   griddep_wait();
   if (seg_stopped(d)) return;
   seg_edge_sample(d, d.ctl->t);
@@ -73,7 +82,7 @@ __global__ void k_seg_edge_sample(Dev d) {
 // ------------------------------------------------------------------ persistent step
 // All steps in one cooperative launch: two grid barriers per step.
 template <bool OUT, bool TYPES>
-__device__ __forceinline__ void seg_persistent(const Dev& d, GridSync* gs, int n_steps, long long limit,
+__device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, int n_steps, long long limit,
                                                unsigned char* smem) {
   int* err = &d.ctl->err;
   const int t0 = (int)*(volatile long long*)&d.ctl->t;
@@ -88,7 +97,7 @@ __device__ __forceinline__ void seg_persistent(const Dev& d, GridSync* gs, int n
   }
 }
 
-__global__ void __launch_bounds__(1024, 1) k_seg_persistent(Dev d, GridSync* gs, int n_steps, long long limit) {
+__global__ void __launch_bounds__(1024, 1) k_seg_persistent(SegDev d, GridSync* gs, int n_steps, long long limit) {
   extern __shared__ __align__(16) unsigned char seg_smem[];
   if (*(volatile int*)&d.ctl->grow) return;
   const bool out = d.emis || d.tt_sum;
@@ -105,9 +114,9 @@ static size_t seg_persistent_smem(int threads) {
   return std::max<size_t>(kSegSmemBytes, (size_t)(threads / 32) * kSegWarpBytes);
 }
 
-cudaError_t launch_seg_persistent(const Dev& d, GridSync* gs, int blocks, int threads, int n_steps, long long limit,
+cudaError_t launch_seg_persistent(const SegDev& d, GridSync* gs, int blocks, int threads, int n_steps, long long limit,
                                   cudaStream_t s) {
-  Dev dd = d;
+  SegDev dd = d;
   void* args[] = {&dd, &gs, &n_steps, &limit};
   return cudaLaunchCooperativeKernel((const void*)k_seg_persistent, dim3(blocks), dim3(threads), args,
                                      seg_persistent_smem(threads), s);
@@ -131,7 +140,7 @@ bool seg_persistent_fits(int threads, int per_sm) {
 // ------------------------------------------------------------------ between the forms
 // Static lane records from the link records and class parameters (after creation, and
 // whenever the class parameters change).
-__global__ void k_seg_lane_stat(Dev d, LaneStat* out, uint32_t* info_out, int32_t* to) {
+__global__ void k_seg_lane_stat(SegDev d, LaneStat* out, uint32_t* info_out, int32_t* to) {
   GRID_STRIDE(lg, d.n_lanes) {
     const int e = d.lane_link[lg];
     const LinkRec L = d.links[e];
@@ -145,14 +154,14 @@ __global__ void k_seg_lane_stat(Dev d, LaneStat* out, uint32_t* info_out, int32_
   }
 }
 
-void launch_seg_lane_stat(const Dev& d, int grid, cudaStream_t s) {
+void launch_seg_lane_stat(const SegDev& d, int grid, cudaStream_t s) {
   k_seg_lane_stat<<<grid, 256, 0, s>>>(d, const_cast<LaneStat*>(d.lstat), const_cast<uint32_t*>(d.sinfo),
                                       const_cast<int32_t*>(d.slot_to));
 }
 
 // the last lane change of a vehicle rides in the high bits of its movement class while the
 // sorted form is laid out
-__global__ void k_seg_mark(Dev d) {
+__global__ void k_seg_mark(SegDev d) {
   const int nA = d.ctl->nA;
   GRID_STRIDE(s, nA) {
     const int c = d.adec[s];
@@ -160,14 +169,14 @@ __global__ void k_seg_mark(Dev d) {
   }
 }
 
-__global__ void k_seg_unmark(Dev d) {
+__global__ void k_seg_unmark(SegDev d) {
   const int nA = d.ctl->nA;
   GRID_STRIDE(s, nA) d.A.mv[s] &= 3;
 }
 
 // Place the sorted vehicles into the segments (the fit is checked first: a state that does
 // not fit sets Ctl::grow and is laid out again in larger segments).
-__global__ void k_seg_place_lanes(Dev d) {
+__global__ void k_seg_place_lanes(SegDev d) {
   GRID_STRIDE(g, d.n_slots) {
     const uint32_t info = d.sinfo[g];
     int next = INT_MAX;
@@ -199,7 +208,7 @@ __global__ void k_seg_place_lanes(Dev d) {
   }
 }
 
-__global__ void k_seg_place(Dev d) {
+__global__ void k_seg_place(SegDev d) {
   if (d.ctl->grow) return;
   const int nB = d.ctl->nB;
   const int t = (int)d.ctl->t;
@@ -225,7 +234,7 @@ void launch_count(const Dev& d, int grid, cudaStream_t s);
 
 // Buffer A -> segments.  The lane counts are made anew, so that it does not matter whether
 // the counts of A are current.
-cudaError_t launch_seg_import(const Dev& d, int grid, cudaStream_t s) {
+cudaError_t launch_seg_import(const SegDev& d, int grid, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(d.cnt, 0, (size_t)d.n_lanes * 4, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.rear2, 0, (size_t)d.n_slots * 2 * sizeof(RearRec), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.best2, 0xFF, (size_t)d.n_slots * 8, s);
@@ -243,7 +252,7 @@ cudaError_t launch_seg_import(const Dev& d, int grid, cudaStream_t s) {
 
 // Every vehicle of the segments, a group of lanes per warp: f(record, link).
 template <typename F>
-__device__ __forceinline__ void seg_for_each(const Dev& d, F f) {
+__device__ __forceinline__ void seg_for_each(const SegDev& d, F f) {
   const int wl = threadIdx.x & 31;
 #pragma unroll 1
   GRID_STRIDE(g, d.n_slots) {
@@ -271,7 +280,7 @@ __device__ __forceinline__ void seg_for_each(const Dev& d, F f) {
 }
 
 // Segments -> buffer A (slots in no particular order; its counts follow by k_count).
-__global__ void k_seg_export(Dev d) {
+__global__ void k_seg_export(SegDev d) {
   if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->active_last = d.ctl->nact[((int)d.ctl->t + 1) & 1];
   seg_for_each(d, [&](const VehRec& r, int e) {
     const unsigned m = __activemask();
@@ -292,7 +301,7 @@ __global__ void k_seg_export(Dev d) {
   });
 }
 
-cudaError_t launch_seg_export(const Dev& d, int grid, cudaStream_t s) {
+cudaError_t launch_seg_export(const SegDev& d, int grid, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(&d.ctl->nA, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.cnt, 0, (size_t)d.n_lanes * 4, s);
   if (e != cudaSuccess) return e;
@@ -302,7 +311,7 @@ cudaError_t launch_seg_export(const Dev& d, int grid, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ readers
-__global__ void k_seg_state_out(Dev d, int32_t* link, int32_t* lane, int32_t* cursor, float* x, float* v,
+__global__ void k_seg_state_out(SegDev d, int32_t* link, int32_t* lane, int32_t* cursor, float* x, float* v,
                                 int8_t* dec) {
   seg_for_each(d, [&](const VehRec& r, int e) {
     const int i = r.vid;
@@ -316,13 +325,13 @@ __global__ void k_seg_state_out(Dev d, int32_t* link, int32_t* lane, int32_t* cu
   });
 }
 
-void launch_seg_state_out(const Dev& d, int grid, cudaStream_t s, int32_t* link, int32_t* lane, int32_t* cursor,
+void launch_seg_state_out(const SegDev& d, int grid, cudaStream_t s, int32_t* link, int32_t* lane, int32_t* cursor,
                           float* x, float* v, int8_t* dec) {
   k_seg_state_out<<<grid, 256, 0, s>>>(d, link, lane, cursor, x, v, dec);
 }
 
 // k_observe on the segments.
-__global__ void k_seg_observe(Dev d, const double* target, double* res, double* p_out) {
+__global__ void k_seg_observe(SegDev d, const double* target, double* res, double* p_out) {
   double acc = 0.0;
   seg_for_each(d, [&](const VehRec& r, int) {
     const double p = prefix_len(d, r.vid, r.ri - d.roff[r.vid]) + (double)r.x;
@@ -350,7 +359,7 @@ __global__ void k_seg_observe(Dev d, const double* target, double* res, double* 
   }
 }
 
-void launch_seg_observe(const Dev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out) {
+void launch_seg_observe(const SegDev& d, int grid, cudaStream_t s, const double* target, double* res, double* p_out) {
   k_seg_observe<<<grid, 256, 0, s>>>(d, target, res, p_out);
 }
 
@@ -383,7 +392,7 @@ static int seg_move_blocks(K kern) {
 
 // Grids: one resident wave, or what the lanes and groups need.  Where the groups outnumber the
 // warps of a resident move phase, their runs are packed (Dev::packed = those warps).
-void seg_grids(Dev& d, int sm_count) {
+void seg_grids(SegDev& d, int sm_count) {
   int f[4] = {};
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f[0], k_seg_front<false, false>, 256, 0);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f[1], k_seg_front<true, false>, 256, 0);
@@ -399,13 +408,13 @@ void seg_grids(Dev& d, int sm_count) {
   for (int v = 0; v < 5; v++) d.seg_move_grid[v] = std::max(1, std::min(d.n_slots / 32 * d.parts, std::max(1, m[v]) * sm_count));
 }
 
-void launch_seg_front(const Dev& d, cudaStream_t s) {
+void launch_seg_front(const SegDev& d, cudaStream_t s) {
   if (d.tape) launch_pdl3(k_seg_front<false, true>, d.seg_front_grid[2], 256, 0, s, d);
   else if (d.vtype) launch_pdl3(k_seg_front<true, false>, d.seg_front_grid[1], 256, 0, s, d);
   else launch_pdl3(k_seg_front<false, false>, d.seg_front_grid[0], 256, 0, s, d);
 }
 
-void launch_seg_move(const Dev& d, cudaStream_t s) {
+void launch_seg_move(const SegDev& d, cudaStream_t s) {
   const bool out = d.emis || d.tt_sum;
   const int v = d.tape ? 4 : (out ? 1 : 0) + (d.vtype ? 2 : 0);
   const int grid = d.seg_move_grid[v];
@@ -418,14 +427,14 @@ void launch_seg_move(const Dev& d, cudaStream_t s) {
   }
 }
 
-void launch_seg_step(const Dev& d, int grid, cudaStream_t s) {
+void launch_seg_step(const SegDev& d, int grid, cudaStream_t s) {
   if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
   launch_seg_front(d, s);
   launch_seg_move(d, s);
 }
 
 // The same step with an event after either phase; ms[0] front (and edge sample), ms[1] move.
-cudaError_t launch_seg_steps_timed(const Dev& d, int grid, cudaStream_t s, int n, float* ms) {
+cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, int n, float* ms) {
   cudaEvent_t ev[3];
   for (int k = 0; k < 3; k++) {
     cudaError_t e = cudaEventCreate(&ev[k]);

@@ -82,7 +82,7 @@ static_assert(4 * (kSegSmemBytes + 1024) <= 228 * 1024, "four blocks per SM");
 // staging area.
 __device__ __forceinline__ bool seg_big(int vehicles, int lanes) { return vehicles + lanes >= kSegN; }
 
-__device__ __forceinline__ bool seg_stopped(const Dev& d) {
+__device__ __forceinline__ bool seg_stopped(const SegDev& d) {
   return (*(volatile int*)&d.ctl->err & kErrTimeout) != 0 || *(volatile int*)&d.ctl->grow != 0;
 }
 
@@ -120,7 +120,7 @@ __device__ __forceinline__ int seg_turn(const LinkNext& a, const LinkNext& b) {
 
 // Eq. 7 parameters of trip vid on a lane (types: its vehicle's).
 template <bool TYPES>
-__device__ __forceinline__ void seg_par(const Dev& d, const float4& A, const float4& B, int vid, ClassPar& P,
+__device__ __forceinline__ void seg_par(const SegDev& d, const float4& A, const float4& B, int vid, ClassPar& P,
                                         float& v0) {
   if (TYPES) {
     const int ty = d.vtype[vid];
@@ -135,7 +135,7 @@ __device__ __forceinline__ void seg_par(const Dev& d, const float4& A, const flo
 // acc_front on the records of this form: om is the vehicle's free-road term, nlb its next
 // link's lanes, rin / tag the rear records of step t.
 template <bool TYPES>
-__device__ __forceinline__ float seg_acc_front(const Dev& d, const RearRec* rin, unsigned tag, float len,
+__device__ __forceinline__ float seg_acc_front(const SegDev& d, const RearRec* rin, unsigned tag, float len,
                                                const ClassPar& P, float om, int vid, int nlb, int lane, float x,
                                                float v, bool closed, TapeForm* f, int* gt = nullptr,
                                                bool* lead = nullptr, float* room = nullptr) {
@@ -205,8 +205,8 @@ struct SegPack {
 
 // Whether link (its lane's thread asks) is left to a whole block, and whether the step may
 // begin: it brings a link at most one vehicle per lane, which must fit.
-__device__ __forceinline__ bool seg_check_link(const Dev& d, int g, int lane, int lanes, int total, int t) {
-  if (total + lanes > kSegBig || total + lanes > d.lane_seg[g].y)
+__device__ __forceinline__ bool seg_check_link(const SegDev& d, int g, int lane, int lanes, int total, int cap, int t) {
+  if (total + lanes > kSegBig || total + lanes > cap)
     atomicMax(&d.ctl->grow, total + lanes > kSegBig ? 2 : 1);
   const bool big = seg_big(total, lanes);
   if (big && lane == 0) d.big_links[atomicAdd(&d.ctl->n_bigl[t & 1], 1)] = d.lstat[g].link;
@@ -218,7 +218,7 @@ __device__ __forceinline__ bool seg_check_link(const Dev& d, int g, int lane, in
 // compacted, then cut greedily into at most 32 lanes and `most` vehicles.  On a sparse
 // network a run gathers the few busy links of many slots.  One pair of list allocations per
 // block: thousands of additions to one counter would outlast the rest of the phase.
-__device__ __forceinline__ void seg_pack(const Dev& d, SegPack* packs, int base, int most, int t) {
+__device__ __forceinline__ void seg_pack(const SegDev& d, SegPack* packs, int base, int most, int t) {
   const int wl = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   SegPack& P = packs[warp];
   base += warp * kPackSlots;
@@ -233,7 +233,7 @@ __device__ __forceinline__ void seg_pack(const Dev& d, SegPack* packs, int base,
     const int cnt = (int)(r >> 16), end = (int)(r & 0xffffu) + cnt;
     const int total = __shfl_sync(0xffffffffu, end, (wl + lanes - 1 - lane) & 31);
     const bool due = __shfl_sync(0xffffffffu, q <= t ? 1 : 0, (wl - lane) & 31) != 0;
-    const bool big = total > 0 && lane_ok && seg_check_link(d, g, lane, lanes, total, t);
+    const bool big = total > 0 && lane_ok && seg_check_link(d, g, lane, lanes, total, d.lane_seg[g].y, t);
     const bool act = lane_ok && !big && (total > 0 || due);
     const unsigned m = __ballot_sync(0xffffffffu, act);
     const int inc = warp_inclusive(act ? cnt : 0);
@@ -293,7 +293,7 @@ __device__ __forceinline__ void seg_pack(const Dev& d, SegPack* packs, int base,
 // arrays, front record and link record, rear record of the next lane.  The runs of the move
 // phase are packed by the last blocks of the grid, which have fewer slots.
 template <bool TYPES, bool TAPE>
-__device__ __forceinline__ void seg_front(const Dev& d, SegPack* packs, int t) {
+__device__ __forceinline__ void seg_front(const SegDev& d, SegPack* packs, int t) {
   const RearRec* rin = d.rear2 + (size_t)(t & 1) * d.n_slots;
   const unsigned tag = (unsigned)t + 1u;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -315,18 +315,28 @@ __device__ __forceinline__ void seg_front(const Dev& d, SegPack* packs, int t) {
   GRID_STRIDE(g, d.n_slots) {
     const uint32_t r = d.rng[g];
     const int cnt = (int)(r >> 16), end = (int)(r & 0xffffu) + cnt;
+    // (few groups: the slot's other arrays are loaded along with its range; many: only for
+    // the slots with vehicles)
+    const float4* ls = reinterpret_cast<const float4*>(d.lstat + g);
     uint32_t info = 0;
-    if (!d.packed) {
+    int2 sg = make_int2(0, 0);
+    float4 A, B;
+    if (!d.packed || cnt) {
       info = d.sinfo[g];
-      const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1;
+      sg = d.lane_seg[g];
+      B = ls[1];
+      A = ls[0];
+    }
+    const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1, ctrl = ctrl_of(info);
+    if (!d.packed) {
       const int total = __shfl_sync(0xffffffffu, end, (wl + lanes - 1 - lane) & 31);
-      const bool big = total > 0 && seg_check_link(d, g, lane, lanes, total, t);
+      const bool big = total > 0 && seg_check_link(d, g, lane, lanes, total, sg.y, t);
       // parts of about the same number of vehicles, 16 at least
       const int w = big ? 0 : cnt, all = __reduce_add_sync(0xffffffffu, w);
       unsigned long long cuts = ~0ull;
       if (all > 16 && d.parts > 1) {
         const int most = max(16, (all + d.parts - 1) / d.parts);
-        const bool in = ctrl_of(info) != kCtrlPad;
+        const bool in = ctrl != kCtrlPad;
         const int inc = warp_inclusive(w);
         cuts = 0;
         int ja = 0;
@@ -339,14 +349,8 @@ __device__ __forceinline__ void seg_front(const Dev& d, SegPack* packs, int t) {
       if (wl == 0) d.cuts[g >> 5] = cuts;
     }
     if (cnt == 0) continue;
-    if (d.packed) info = d.sinfo[g];
-    const int2 sg = d.lane_seg[g];
-    const int lane = (int)(info & 7u), ctrl = (int)(info >> 6 & 3u);
     const VehRec f = seg_load(d.rec + sg.x + end - 1);
-    const float4* ls = reinterpret_cast<const float4*>(d.lstat + g);
-    const float4 B = ls[1];
     const int e = __float_as_int(B.w);
-    const float4 A = ls[0];
     LinkRec L;
     if (ctrl != kCtrlNone) L = d.links[e];
     ClassPar P;
@@ -441,7 +445,7 @@ __device__ __forceinline__ int seg_upper(const SM& S, int s0, int s1, float x, i
 // acceptance = positive lead and lag gaps and both the changer's and the new follower's
 // accelerations >= -b_safe.
 template <typename SM, bool TYPES, bool TAPE>
-__device__ __forceinline__ void seg_decide(const Dev& d, SM& S, int i, const RearRec* rin, unsigned tag) {
+__device__ __forceinline__ void seg_decide(const SegDev& d, SM& S, int i, const RearRec* rin, unsigned tag) {
   const int j = S.jo[i];
   const float4 A = S.la[j], B = S.lb[j];
   const unsigned info = __float_as_uint(B.z);
@@ -553,7 +557,7 @@ __device__ __forceinline__ void seg_decide(const Dev& d, SM& S, int i, const Rea
 // lane is sorted, so the scan covers a window around x that holds every vehicle that can
 // pass the test.
 template <typename SM, bool TYPES>
-__device__ __forceinline__ bool seg_cancelled(const Dev& d, const SM& S, int i, int j, int j2, int first, int last) {
+__device__ __forceinline__ bool seg_cancelled(const SegDev& d, const SM& S, int i, int j, int j2, int first, int last) {
   const float s0c = S.la[j].w;
   const float x = S.x[i];
   const int vid = S.vid[i];
@@ -588,7 +592,7 @@ __device__ __forceinline__ bool seg_cancelled(const Dev& d, const SM& S, int i, 
 // in this step, if that space is at least s0 + vehicle length.  Called by the thread of the
 // link's first lane j0.
 template <typename SM, bool OUT, bool TYPES>
-__device__ __noinline__ void seg_depart(const Dev& d, SM& S, int n, int j0, int t, int* count) {
+__device__ __noinline__ void seg_depart(const SegDev& d, SM& S, int n, int j0, int t, int* count) {
   const float4 B = S.lb[j0];
   const int e = __float_as_int(B.w);
   const int lanes = (int)(__float_as_uint(B.z) >> 3 & 7u) + 1;
@@ -641,7 +645,7 @@ __device__ __noinline__ void seg_depart(const Dev& d, SM& S, int n, int j0, int 
 // thread knows of its lane goes to shared memory at once: kept in registers over the whole
 // run it spilled, and next to the staging areas the L1 is too small to hold the spills.
 template <int NT, typename SM, bool OUT, bool TYPES, bool TAPE>
-__device__ __forceinline__ void seg_run(const Dev& d, SM& S, const SegLane& ln, int nl, int t,
+__device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& ln, int nl, int t,
                                         int* count) {
   const int tid = NT == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   const int nt = NT == 32 ? 32 : (int)blockDim.x;
@@ -1038,7 +1042,7 @@ __device__ __forceinline__ void seg_run(const Dev& d, SM& S, const SegLane& ln, 
 }
 
 // What the thread of slot g needs (g < 0: none).
-__device__ __forceinline__ SegLane seg_lane(const Dev& d, int g, int t) {
+__device__ __forceinline__ SegLane seg_lane(const SegDev& d, int g, int t) {
   SegLane ln;
   ln.on = ln.ext = ln.due = false;
   ln.g = g;
@@ -1048,42 +1052,39 @@ __device__ __forceinline__ SegLane seg_lane(const Dev& d, int g, int t) {
   ln.lb = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(-1));
   if (g < 0) return ln;
   ln.on = true;
+  // one level of loads that depend on nothing
   const uint32_t r = d.rng[g];
   const unsigned long long bk = d.best2[g];
-  const int q = d.qnext[g];
+  const int q = d.qnext[g], tail = d.stail[g];
   const float4* ls = reinterpret_cast<const float4*>(d.lstat + g);
   ln.lb = ls[1];
   ln.la = ls[0];
   ln.seg = d.lane_seg[g].x;
+  ln.to = d.slot_to[g];
+  ln.fr = d.fres[g];
   ln.start = (int)(r & 0xffffu);
   ln.cnt = (int)(r >> 16);
   const unsigned info = __float_as_uint(ln.lb.z);
-  if (ln.cnt) {   // (an empty lane's record is an older step's)
-    ln.fr = d.fres[g];
-    if ((info >> 6 & 3u) == (unsigned)kCtrlStop) ln.to = d.slot_to[g];
-    if (ln.fr.y & kSegCand) {
-      const unsigned long long k = d.best2[ln.fr.y >> 4];
-      if (epoch_current(k, t) && ((unsigned)k & 0xFFFFu) == ((info & 7u) << 8 | (info >> 16 & 255u)))
-        ln.fr.y |= kSegWon;
-    }
-    ln.fr.y &= kSegWon | 15;
-  } else if ((info >> 6 & 3u) == (unsigned)kCtrlStop) {
-    ln.to = d.slot_to[g];
-  }
+  if (ln.cnt == 0) ln.fr.y = 0;   // an empty lane's record is an older step's
   if (epoch_current(bk, t)) {
     ln.ext = true;
-    ln.src = d.nin_slot[d.tail_in[__float_as_int(ln.lb.w)] + (int)((unsigned)bk & 255u)] +
-             (int)((unsigned)bk >> 8 & 255u);
+    ln.src = d.nin_slot[tail + (int)((unsigned)bk & 255u)] + (int)((unsigned)bk >> 8 & 255u);
   }
+  if (ln.fr.y & kSegCand) {
+    const unsigned long long k = d.best2[ln.fr.y >> 4];
+    if (epoch_current(k, t) && ((unsigned)k & 0xFFFFu) == ((info & 7u) << 8 | (info >> 16 & 255u)))
+      ln.fr.y |= kSegWon;
+  }
+  ln.fr.y &= kSegWon | 15;
   ln.due = q <= t;
   return ln;
 }
 
 // A link without vehicles or departures that crossing vehicles may have entered, by one
 // thread: at most one vehicle per lane, already in order.
-__device__ __forceinline__ void seg_enter(const Dev& d, int e, int t) {
+__device__ __forceinline__ void seg_enter(const SegDev& d, int e, int t) {
   const int g0 = d.lslot[e];
-  const int seg = d.lane_seg[g0].x, tail = d.tail_in[e], to = d.slot_to[g0];
+  const int seg = d.lane_seg[g0].x, tail = d.stail[g0], to = d.slot_to[g0];
   const unsigned info = d.sinfo[g0];
   const int lanes = (int)(info >> 3 & 7u) + 1;
   RearRec* rout = d.rear2 + (size_t)((t + 1) & 1) * d.n_slots;
@@ -1108,7 +1109,7 @@ __device__ __forceinline__ void seg_enter(const Dev& d, int e, int t) {
 // the empty links that vehicles enter, 32 per warp.  Units of one run per warp are dealt to
 // the blocks after the big links (a unit each); few runs spread over all blocks.
 template <bool OUT, bool TYPES, bool TAPE>
-__device__ __forceinline__ void seg_move(const Dev& d, unsigned char* smem, int t) {
+__device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, int t) {
   const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
   __shared__ int s_cn[4];
   if (threadIdx.x < 4) s_cn[threadIdx.x] = 0;
@@ -1146,13 +1147,13 @@ __device__ __forceinline__ void seg_move(const Dev& d, unsigned char* smem, int 
       jend = p < 7 ? min(32, (int)(cuts >> (8 * p) & 255u)) : 32;
       if (ja >= jend) continue;
       g = grp * 32 + wl;
-      if (ctrl_of(d.sinfo[g]) == kCtrlPad) g = -1;
     }
 #pragma unroll 1
     do {
       SegLane ln = seg_lane(d, g, t);
-      if (!d.packed) {   // links left to whole blocks
+      if (!d.packed) {   // empty slots, links left to whole blocks
         const unsigned info = __float_as_uint(ln.lb.z);
+        if (ctrl_of(info) == kCtrlPad) ln.on = false;
         const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1;
         if (seg_big(__shfl_sync(0xffffffffu, ln.start + ln.cnt, (wl + lanes - 1 - lane) & 31), lanes)) ln.on = false;
       }
@@ -1161,7 +1162,7 @@ __device__ __forceinline__ void seg_move(const Dev& d, unsigned char* smem, int 
       int jb = jend;
       if (__reduce_add_sync(0xffffffffu, w) > kSegN) {
         const unsigned info = __float_as_uint(ln.lb.z);
-        jb = min(jb, seg_run_end(ja, warp_inclusive(w), (int)(info & 7u), (int)(info >> 3 & 7u) + 1, g >= 0, kSegN));
+        jb = min(jb, seg_run_end(ja, warp_inclusive(w), (int)(info & 7u), (int)(info >> 3 & 7u) + 1, ln.on || wl < jend, kSegN));
         ln.on = ln.on && wl < jb;
       }
       if (__any_sync(0xffffffffu, ln.on && (ln.cnt || ln.ext || ln.due)))

@@ -11,10 +11,15 @@ namespace gbt {
 // The step kernels are launched with programmatic stream serialization: a kernel's
 // launch is prepared while the one before it in the stream runs, and the kernel waits
 // here, before its first read, until that grid has completed and its writes are
-// visible.  (Without such a launch the wait returns at once.)  No kernel triggers its
-// dependents early: waiting blocks would hold registers and shared memory that the
-// running kernel's blocks use (measured slower).
+// visible.  (Without such a launch the wait returns at once.)  Only on small networks does a
+// kernel let its dependents in early (griddep_next_small): elsewhere waiting blocks would hold
+// registers and shared memory that the running kernel's blocks use (measured slower).
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+constexpr int kSmallLanes = 2048;
+__device__ __forceinline__ void griddep_next_small(const Dev& d) {
+  if (d.n_lanes < kSmallLanes) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 // Arrival index of this vehicle in lane g's count for the next occupancy rebuild.
 // Neighbouring threads mostly hold vehicles of the same lane (the sorted order), so
