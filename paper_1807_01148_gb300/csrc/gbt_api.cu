@@ -52,6 +52,7 @@ void launch_fw_final_time(const double* t0, const double* x, const double* cap, 
                           int n, cudaStream_t s);
 void launch_compact_routes(const int32_t* roff, const int32_t* rlen, const int32_t* src, const int32_t* new_off,
                            int32_t* dst, int n, cudaStream_t s);
+void launch_seg_pack(const SegDev& d, cudaStream_t s);
 void launch_seg_step(const SegDev& d, int grid, cudaStream_t s);
 cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, int n, float* ms);
 cudaError_t launch_seg_import(const SegDev& d, int grid, cudaStream_t s);
@@ -91,6 +92,7 @@ struct NvtxRange {
 // Steps captured into one graph where several follow each other: what a graph launch costs
 // between two steps (about 2 us) is then paid once per kUnroll steps.
 constexpr int kUnroll = 8;
+static_assert(kUnroll <= kPackSteps, "a graph packs its runs once");
 struct StepGraph {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -150,6 +152,7 @@ struct sim_handle {
   // captured steps: one, kUnroll in a row, one with the per-edge sample kernel (launched at
   // sampling instants only); the taping ones of the adjoint
   StepGraph step1, step8, samp1, tape1, tape8;
+  int pack_age = 1 << 20;   // steps since the runs were packed
   int steps_run = 0, tape_steps_run = 0;   // steps made with the present ones
   bool graph_dirty = true;
   // class parameters (host copies) and the adjoint's tape
@@ -252,15 +255,17 @@ int upload(sim_handle* h, T** p, const T* src, size_t n) {
 // either way): the segments on any network.  Measured, us per step, sorted -> segments: 20 x
 // 20 grid (3,040 lanes, 2,050 vehicles) 41.6 -> 22.2; town of 6,700 lanes 16.3 -> 8.6 (with its
 // share of planning); district of 42,000 lanes with outputs and trucks 78 -> 71.
-// Not in the segments: networks with more groups of lanes than resident warps of the move
-// phase (from kSegLanesMost lanes on; metro, 782,000 lanes and 2.11M vehicles: 247 -> 253),
-// and those where links longer than a staged chunk carry most of the road, for which the
-// sorted form has its big-chunk kernel (1,000 queues of 570 vehicles: 118 against 122).
-constexpr int kSegLanes = 2048, kSegLanesMost = 150000;
+// On networks with more groups of lanes than resident warps of the move phase, in packed
+// lists (SegDev::packed; us per step): 64 copies of a grid 76.8 -> 64.5; metro, 782,000 lanes,
+// 2.11M vehicles 274 -> 269 and, in the persistent launch with 500,000, 89 -> 78.
+// Not in the segments: networks where links longer than a staged chunk carry most of the
+// road, for which the sorted form has its big-chunk kernel (1,000 queues of 570 vehicles: 118
+// against 122).
+constexpr int kSegLanes = 2048;
 
 bool seg_possible(const sim_handle* h) { return !h->seg_off && !h->long_route; }
 
-bool seg_sized(const sim_handle* h) { return !h->d.chunk_split && h->n_lanes <= kSegLanesMost; }
+bool seg_sized(const sim_handle* h) { return !h->d.chunk_split; }
 
 bool seg_wanted(const sim_handle* h) {
   return seg_possible(h) && seg_sized(h) &&
@@ -364,10 +369,9 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   get(&d.nin_slot, (size_t)nl, nin.data());
   get(&d.qnext, ns);
   get(&d.big_links, (size_t)std::max(1, n_big));
-  get(&d.tl, ns);
-  get(&d.runs, (size_t)nl);
+  get(&d.tl, (size_t)nl * 32);   // a run has one link at least
   get(&d.late, (size_t)nl);
-  get(&d.claim, (size_t)nl);
+  get(&d.listed, (size_t)nl);
   get(&d.cuts, ns / 32);
   if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(h, SIM_ECUDA, "segment tables");
   h->seg_building = false;
@@ -403,6 +407,7 @@ int seg_from_sorted(sim_handle* h) {
     const int grow = h->mirror->c.grow;
     if (!grow) {
       h->seg = true;
+      h->pack_age = 1 << 20;
       return SIM_OK;
     }
     if (grow == 2 || attempt == 1) {
@@ -1367,10 +1372,13 @@ int sim_read_routes(sim_handle* h, int32_t* offsets, int32_t* links) {
 
 namespace {
 
-// Capture n steps in the present form into G, if it is not there already.
+// Capture n steps in the present form into G, if it is not there already.  Several steps begin
+// with the packing of the runs; before a single one it is a launch of its own (pack_runs): a
+// second graph with it lengthened the first steps of a large network by 150 us.
 int capture_steps(sim_handle* h, StepGraph& G, const SegDev& d, int n) {
   if (G.exec) return SIM_OK;
   CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  if (h->seg && d.packed && n > 1) launch_seg_pack(d, h->cap_stream);
   for (int k = 0; k < n; k++) {
     if (h->seg) launch_seg_step(d, h->grid, h->cap_stream);
     else launch_step(d, h->grid, h->has_stop, h->cap_stream);
@@ -1385,6 +1393,14 @@ int capture_steps(sim_handle* h, StepGraph& G, const SegDev& d, int n) {
   return SIM_OK;
 }
 
+// Before a single step: the packing, if the lists are too old; returns the launches it took.
+int pack_runs(sim_handle* h) {
+  const bool pack = h->seg && h->d.packed && h->pack_age >= kPackSteps;
+  if (pack) launch_seg_pack(h->d, h->stream);
+  h->pack_age = pack ? 1 : std::min(h->pack_age + 1, 1 << 20);
+  return pack ? 1 : 0;
+}
+
 // n steps as graphs: kUnroll at a time, then one by one.  Without tape: the plain steps of
 // sim_step (no edge sample); with it: the adjoint's taping steps.
 int enqueue_graph_steps(sim_handle* h, int n, bool tape, bool count) {
@@ -1395,7 +1411,9 @@ int enqueue_graph_steps(sim_handle* h, int n, bool tape, bool count) {
   if (dirty || form != h->seg) {
     g1.drop();
     g8.drop();
-    if (!tape) h->samp1.drop();
+    if (!tape) {
+      h->samp1.drop();
+    }
     steps = 0;
     dirty = false;
     form = h->seg;
@@ -1411,10 +1429,13 @@ int enqueue_graph_steps(sim_handle* h, int n, bool tape, bool count) {
     // (the longer graph only once enough steps were made to pay for its capture)
     const bool many = n - k >= kUnroll && (g8.exec || n >= 8 * kUnroll || steps >= 8 * kUnroll);
     const int m = many ? kUnroll : 1;
-    StepGraph& G = m > 1 ? g8 : g1;
+    StepGraph& G = many ? g8 : g1;
     if (int rc = capture_steps(h, G, d, m)) return rc;
+    int pack = 0;
+    if (many) h->pack_age = m;
+    else pack = pack_runs(h);
     CK(cudaGraphLaunch(G.exec, h->stream));
-    if (count) h->launches += (long long)G.nodes;
+    if (count) h->launches += (long long)G.nodes + pack;
     k += m;
     steps = std::min(steps + m, 1 << 20);
   }
@@ -1464,6 +1485,7 @@ int enqueue_steps(sim_handle* h, long long t0, int n_steps) {
     if (h->pexec) CK(cudaGraphLaunch(h->pexec, h->stream));
     else CK(launch(h->stream));
     h->launches += 1;
+    h->pack_age = 1 << 20;
     return SIM_OK;
   }
   const long long every = h->d.acc_u ? h->d.samp_every : 0;
@@ -1471,6 +1493,7 @@ int enqueue_steps(sim_handle* h, long long t0, int n_steps) {
     if (every > 0 && (t0 + s) % every == 0) {   // a sampling instant
       if (int rc = enqueue_graph_steps(h, 0, false, true)) return rc;
       if (int rc = capture_steps(h, h->samp1, h->d, 1)) return rc;
+      h->launches += pack_runs(h);
       CK(cudaGraphLaunch(h->samp1.exec, h->stream));
       h->launches += (long long)h->samp1.nodes;
       s++;
@@ -1567,6 +1590,7 @@ int sim_step_timed(sim_handle* h, int32_t n_steps, float* kernel_ms) {
     const long long t_end = h->t_host + n_steps;
     float ms[2] = {0.0f, 0.0f};
     CK(launch_seg_steps_timed(h->d, h->grid, h->stream, n_steps, ms));
+    h->pack_age = 1 << 20;
     kernel_ms[kKFront] = ms[0];
     kernel_ms[kKChunk] = ms[1];
     if (int rc = check_device(h)) return rc;
@@ -1986,7 +2010,7 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
   }
   // both passes in the segment form, on any network, if its memory is there (the working
   // memory above comes first)
-  if (seg_possible(h) && (rc = seg_from_sorted(h))) {
+  if ((rc = seg_possible(h) ? seg_from_sorted(h) : seg_to_sorted(h))) {
     release();
     return rc;
   }

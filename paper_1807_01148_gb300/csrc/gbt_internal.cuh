@@ -152,8 +152,12 @@ struct Ctl {
   alignas(128) long long tm;   // step of the running move phase (the front phase's copy of t)
   int grow;                    // the next step does not fit the segments: 1 a segment, 2 a link (no step runs)
   int n_bigl[2];               // links left to whole blocks, by parity of the step
-  alignas(128) int n_tl[2];    // entries of tl, runs and late, by parity of the step
-  int n_run[2], n_late[2];
+  // lists of the packed segment form: runs of step t in half t & 1, what its move phase added
+  // to them, links entered late; the newest packing's runs and t + 1
+  int n_run[2], add_run[2], n_late[2];
+  alignas(128) int pk_run;
+  int pk_step;
+  int pk_veh;                  // vehicles laid out since the last step, else 0
   alignas(128) int nact[2];    // vehicles advanced, by parity of the step
 };
 
@@ -275,9 +279,12 @@ struct Dev {
 // kernel's parameters are copied at its launch (a third more of them cost the sorted form's
 // seven kernels 0.3 to 0.4 us each).  Lanes are numbered by slots: the lanes of whole links
 // fill groups of 32 slots, the rest of a group is left empty.
+constexpr int kPackSteps = 8;   // steps that the packed lists hold for
+
 struct SegDev : Dev {
   VehRec* rec;                     // link e owns cap records from its segment's start on, in (lane, x, vid) order
-  uint32_t* rng;                   // per slot: its vehicles, start relative to the segment | count << 16
+  uint32_t* rng;                   // per slot: its vehicles, start relative to the segment | count << 16 (rng_start,
+                                   // rng_count) | 2 + parity of the step << 30 where a whole block wrote it
   const uint32_t* sinfo;           // per slot: LaneStat::info (control 3: empty slot)
   const int2* lane_seg;            // per slot: its link's segment start and capacity
   const LaneStat* lstat;           // per slot
@@ -291,15 +298,15 @@ struct SegDev : Dev {
   const int32_t* stail;            // per slot: start of its link's tail node's in-links in nin_slot
   const int32_t* nin_slot;         // in-links of every node in ascending id: slot of lane 0
   int n_slots;
-  int packed;                      // runs are packed by the front phase (else they are parts of a group)
+  int packed;                      // runs are packed lists (else parts of a group); the resident warps
   int parts;                       // parts of a group, 1..8
   unsigned long long* cuts;        // per group: first lane of parts 1..7, 8 bits each
   int32_t* qnext;                  // per slot of a lane 0: departure step of its link's queue's head (else INT_MAX)
   int32_t* big_links;              // links with more vehicles than a warp's staging area
-  int32_t* tl;                     // slots of the links with something to do, run after run
-  int2* runs;                      // runs of the move phase: first entry of tl, lanes
-  int32_t* late;                   // empty links that a crossing vehicle may enter
-  int32_t* claim;                  // per link: t + 1 of the step it was last listed in late
+  int32_t* tl;                     // runs of the move phase, 32 entries each: slots of links with something to do,
+                                   // then -1
+  int32_t* late;                   // unlisted links that a crossing vehicle may enter
+  int32_t* listed;                 // per link: Ctl::pk_step of the packing that has it in tl
   int seg_front_grid[4], seg_move_grid[6];
 };
 

@@ -20,17 +20,33 @@ __device__ __forceinline__ void griddep_next(const SegDev& d) {
   if (!d.packed) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Bound by the latency of its dependent loads (range and slot arrays, front record and link
+// record, rear record of the next lane): six blocks of 40 registers per SM.
 template <bool TYPES, bool TAPE>
-__global__ void __launch_bounds__(256) k_seg_front(SegDev d) {
+__global__ void __launch_bounds__(256, 6) k_seg_front(SegDev d) {
   griddep_wait();
   griddep_next(d);
   if (seg_stopped(d)) return;
-  __shared__ SegPack packs[8];
-  seg_front<TYPES, TAPE>(d, packs, (int)d.ctl->t);
+  seg_front<TYPES, TAPE>(d, (int)d.ctl->t);
 }
 
+// The lists of the next kPackSteps steps.  Packed in the front phase of every step they cost as
+// much as the idle lanes that they save (metro, 2.11M vehicles: 253 us per step against 247 in
+// the sorted form); kept for 8 steps, 241.
+__global__ void __launch_bounds__(256) k_seg_pack(SegDev d) {
+  griddep_wait();
+  if (seg_stopped(d)) return;
+  __shared__ SegPack packs[8];
+  seg_pack_all(d, packs, (int)d.ctl->t);
+}
+
+// Bound by instruction issue and load latency together (a quarter of metro, 580,000 vehicles:
+// 42% of issue slots, most stalls on loads, waits within the warp next).  Three blocks of 80
+// registers measured better than four of 64, whose spills miss the little L1 that the staging
+// areas leave: metro, 2.11M vehicles, 4 steps 1,110 -> 1,077 us; 64 grids, 10 steps 670 -> 645;
+// two blocks: 1,269 and 743.
 template <bool OUT, bool TYPES, bool TAPE>
-__global__ void __launch_bounds__(kSegThreads, 4) k_seg_move(SegDev d) {
+__global__ void __launch_bounds__(kSegThreads, 3) k_seg_move(SegDev d) {
   griddep_wait();
   griddep_next(d);
   if (seg_stopped(d)) return;
@@ -52,7 +68,7 @@ __device__ __forceinline__ void seg_edge_sample(const SegDev& d, long long t) {
     const LinkRec L = d.links[e];
     const int g = d.lslot[e];
     const uint32_t last = d.rng[g + L.lanes - 1];
-    const int n = (int)((last & 0xffffu) + (last >> 16));
+    const int n = rng_start(last) + rng_count(last);
     const VehRec* r = d.rec + d.lane_seg[g].x;
     double vs = 0.0;
     for (int q = 0; q < n; q++) vs += (double)r[q].v;
@@ -89,7 +105,11 @@ __device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, in
   for (int step = 0; step < n_steps; step++) {
     const int t = t0 + step;
     if (d.acc_u) seg_edge_sample(d, t);
-    seg_front<TYPES, false>(d, reinterpret_cast<SegPack*>(smem), t);
+    if (d.packed && step % kPackSteps == 0) {
+      seg_pack_all(d, reinterpret_cast<SegPack*>(smem), t);
+      if (!grid_barrier(gs, err, limit)) return;
+    }
+    seg_front<TYPES, false>(d, t);
     if (!grid_barrier(gs, err, limit)) return;
     if (*(volatile int*)&d.ctl->grow) return;   // set before the barrier, the same for every block
     seg_move<OUT, TYPES, false>(d, smem, t);
@@ -187,7 +207,7 @@ __global__ void k_seg_place_lanes(SegDev d) {
       const int lg0 = d.links[e].lane_base;
       const int start = d.lane_start[lg0 + lane] - d.lane_start[lg0];
       const int end = d.lane_start[lg0 + lane + 1] - d.lane_start[lg0];
-      r = (uint32_t)(start & 0xffff) | (uint32_t)(end - start) << 16;   // beyond 16 bits: grow is set
+      r = (uint32_t)(start & 0xffff) | (uint32_t)(end - start & 0x3fff) << 16;   // beyond these bits: grow is set
       if (lane == lanes - 1) {
         const int most = end + lanes;
         if (most > kSegBig) atomicMax(&d.ctl->grow, 2);
@@ -203,7 +223,11 @@ __global__ void k_seg_place_lanes(SegDev d) {
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const int t = (int)d.ctl->t;
-    for (int p = 0; p < 2; p++) d.ctl->n_bigl[p] = d.ctl->n_tl[p] = d.ctl->n_run[p] = d.ctl->n_late[p] = 0;
+    Ctl* c = d.ctl;
+    for (int p = 0; p < 2; p++)
+      c->n_bigl[p] = c->n_run[p] = c->add_run[p] = c->n_late[p] = 0;
+    c->pk_run = c->pk_step = 0;
+    c->pk_veh = c->nB;
     d.ctl->nact[(t + 1) & 1] = d.ctl->active_last;
   }
 }
@@ -238,7 +262,7 @@ cudaError_t launch_seg_import(const SegDev& d, int grid, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(d.cnt, 0, (size_t)d.n_lanes * 4, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.rear2, 0, (size_t)d.n_slots * 2 * sizeof(RearRec), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.best2, 0xFF, (size_t)d.n_slots * 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(d.claim, 0, (size_t)d.n_links * 4, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d.listed, 0, (size_t)d.n_links * 4, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(&d.ctl->grow, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   k_seg_mark<<<grid, 256, 0, s>>>(d);
@@ -259,7 +283,7 @@ __device__ __forceinline__ void seg_for_each(const SegDev& d, F f) {
     const float4 B = reinterpret_cast<const float4*>(d.lstat + g)[1];
     const uint32_t rg = d.rng[g];
     const int e = __float_as_int(B.w);
-    const int start = d.lane_seg[g].x + (int)(rg & 0xffffu), cnt = (int)(rg >> 16);
+    const int start = d.lane_seg[g].x + rng_start(rg), cnt = rng_count(rg);
     const int inc = warp_inclusive(cnt);
     const int pos = inc - cnt, n = __shfl_sync(0xffffffffu, inc, 31);
 #pragma unroll 1
@@ -427,13 +451,20 @@ void launch_seg_move(const SegDev& d, cudaStream_t s) {
   }
 }
 
+// Networks with packed runs: before the first step after the state was laid out, and at least
+// every kPackSteps steps.
+void launch_seg_pack(const SegDev& d, cudaStream_t s) {
+  const int tile = 8 * kPackSlots;
+  launch_pdl3(k_seg_pack, std::max(1, (d.n_slots + tile - 1) / tile), 256, 0, s, d);
+}
+
 void launch_seg_step(const SegDev& d, int grid, cudaStream_t s) {
   if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
   launch_seg_front(d, s);
   launch_seg_move(d, s);
 }
 
-// The same step with an event after either phase; ms[0] front (and edge sample), ms[1] move.
+// The same step with an event after either phase; ms[0] front (with the packing and the edge sample), ms[1] move.
 cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, int n, float* ms) {
   cudaEvent_t ev[3];
   for (int k = 0; k < 3; k++) {
@@ -443,6 +474,7 @@ cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, in
   cudaError_t err = cudaSuccess;
   for (int it = 0; it < n && err == cudaSuccess; it++) {
     cudaEventRecord(ev[0], s);
+    if (d.packed && it % kPackSteps == 0) launch_seg_pack(d, s);
     if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
     launch_seg_front(d, s);
     cudaEventRecord(ev[1], s);

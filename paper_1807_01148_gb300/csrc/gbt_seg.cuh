@@ -6,15 +6,16 @@
 // Lanes are numbered by slots: the lanes of whole consecutive links fill groups of 32, so
 // that the lanes of a link are always threads of one warp.
 //
-//   front  one thread per lane: the links with something to do are packed into runs of
-//          whole links (at most 32 lanes and about 90 vehicles); the lane's front vehicle, its acceleration
-//          behind the rearmost vehicle of the next link's lane or the stop line, its
-//          admission bid and, for a bidder, its record after crossing;
-//   move   a warp per run: its vehicles staged in
-//          shared memory, own-lane Eq. 7, lane-change decisions, conflicts, ballistic
-//          move; then the new order of the same links is written in place.  Vehicles
-//          that won an admission are pulled by the target lane (at most one per lane and
-//          step), departures are appended by the first link's warp.
+//   front  one thread per lane: the lane's front vehicle, its acceleration behind the rearmost
+//          vehicle of the next link's lane or the stop line, its admission bid and, for a
+//          bidder, its record after crossing;
+//   move   a warp per run (whole links, at most 32 lanes and about 90 vehicles: a part of a
+//          group, or on large networks a list of links with something to do that is packed
+//          anew every 8 steps): its vehicles staged in shared memory, own-lane Eq. 7,
+//          lane-change decisions, conflicts, ballistic move; then the new order of the same
+//          links is written in place.  Vehicles that won an admission are pulled by the
+//          target lane (at most one per lane and step), departures are appended by the
+//          first link's warp.
 //
 // The model admits at most one vehicle per lane and step, so a lane's new order is its
 // stayers in their old order plus a few incoming vehicles (lane changers, one crossing or
@@ -31,8 +32,8 @@
 
 namespace gbt {
 
-// A warp stages up to kSegN vehicles; 8 warps of 6.8 KB and 64 registers per thread leave
-// 4 blocks of 256 threads on an SM.  A link with more vehicles is staged by a whole block
+// A warp stages up to kSegN vehicles; 8 warps of 6.8 KB let 4 blocks of 256 threads onto an SM
+// (what a persistent launch may ask for; the kernel of its own takes 3).  A link with more vehicles is staged by a whole block
 // (kSegBig of them in the same memory); one with still more stops the stepping in this form
 // (Ctl::grow = 2) and the sorted form goes on.
 constexpr int kSegN = 96, kSegBig = 1024;
@@ -81,6 +82,10 @@ static_assert(4 * (kSegSmemBytes + 1024) <= 228 * 1024, "four blocks per SM");
 // A link whose vehicles (and one more per lane, and one departure) do not fit a warp's
 // staging area.
 __device__ __forceinline__ bool seg_big(int vehicles, int lanes) { return vehicles + lanes >= kSegN; }
+
+// Fields of SegDev::rng.
+__device__ __forceinline__ int rng_start(uint32_t r) { return (int)(r & 0xffffu); }
+__device__ __forceinline__ int rng_count(uint32_t r) { return (int)(r >> 16 & 0x3fffu); }
 
 __device__ __forceinline__ bool seg_stopped(const SegDev& d) {
   return (*(volatile int*)&d.ctl->err & kErrTimeout) != 0 || *(volatile int*)&d.ctl->grow != 0;
@@ -200,24 +205,27 @@ struct SegPack {
   int32_t slot[kPackSlots];
   uint16_t first[kPackSlots + 1];   // first active lane of each run
   uint8_t last[kPackSlots];         // the active lane is its link's last one
-  int32_t n, n_run, tl0, run0;
+  int32_t n_run, run0;
 };
 
-// Whether link (its lane's thread asks) is left to a whole block, and whether the step may
-// begin: it brings a link at most one vehicle per lane, which must fit.
-__device__ __forceinline__ bool seg_check_link(const SegDev& d, int g, int lane, int lanes, int total, int cap, int t) {
+// For one lane of every link with vehicles: lists it when it is left to a whole block, and
+// stops the step where a segment may run full (the step brings a link at most one vehicle per
+// lane; they must fit, or the move phase does not run).
+__device__ __forceinline__ void seg_check_link(const SegDev& d, int g, int lanes, int total, int cap, int t) {
   if (total + lanes > kSegBig || total + lanes > cap)
     atomicMax(&d.ctl->grow, total + lanes > kSegBig ? 2 : 1);
-  const bool big = seg_big(total, lanes);
-  if (big && lane == 0) d.big_links[atomicAdd(&d.ctl->n_bigl[t & 1], 1)] = d.lstat[g].link;
-  return big;
+  if (seg_big(total, lanes)) d.big_links[atomicAdd(&d.ctl->n_bigl[t & 1], 1)] = d.lstat[g].link;
 }
 
-// Packs the links that have something to do (vehicles, a due departure) into runs of whole
-// links for the move phase, kPackSlots slots per warp of the block: the active lanes are
-// compacted, then cut greedily into at most 32 lanes and `most` vehicles.  On a sparse
-// network a run gathers the few busy links of many slots.  One pair of list allocations per
-// block: thousands of additions to one counter would outlast the rest of the phase.
+// Packs the links that have something to do (vehicles, a departure due before the next
+// packing) into runs of whole links, kPackSlots slots per warp of the block: the active lanes
+// are compacted, then cut greedily into at most 32 lanes and `most` vehicles.  On a sparse
+// network a run gathers the few busy links of many slots.  The lists hold for kPackSteps
+// steps: links that empty stay in them, links that are entered in between are added by the
+// move phase.  One allocation of runs per block: thousands of additions to one counter would
+// outlast the rest.
+constexpr int kPackHorizon = 2 * kPackSteps;
+
 __device__ __forceinline__ void seg_pack(const SegDev& d, SegPack* packs, int base, int most, int t) {
   const int wl = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   SegPack& P = packs[warp];
@@ -230,11 +238,11 @@ __device__ __forceinline__ void seg_pack(const SegDev& d, SegPack* packs, int ba
     const int q = d.qnext[g];
     const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1;
     const bool lane_ok = (info >> 6 & 3u) != (unsigned)kCtrlPad;
-    const int cnt = (int)(r >> 16), end = (int)(r & 0xffffu) + cnt;
+    const int cnt = rng_count(r), end = rng_start(r) + cnt;
     const int total = __shfl_sync(0xffffffffu, end, (wl + lanes - 1 - lane) & 31);
-    const bool due = __shfl_sync(0xffffffffu, q <= t ? 1 : 0, (wl - lane) & 31) != 0;
-    const bool big = total > 0 && lane_ok && seg_check_link(d, g, lane, lanes, total, d.lane_seg[g].y, t);
-    const bool act = lane_ok && !big && (total > 0 || due);
+    const bool due = __shfl_sync(0xffffffffu, q <= t + kPackHorizon ? 1 : 0, (wl - lane) & 31) != 0;
+    const bool act = lane_ok && (total > 0 || due);
+    if (act && lane == 0) d.listed[d.lstat[g].link] = t + 1;
     const unsigned m = __ballot_sync(0xffffffffu, act);
     const int inc = warp_inclusive(act ? cnt : 0);
     if (act) {
@@ -264,73 +272,77 @@ __device__ __forceinline__ void seg_pack(const SegDev& d, SegPack* packs, int ba
   }
   if (wl == 0) {
     P.first[k] = (uint16_t)n;
-    P.n = n;
     P.n_run = k;
   }
   __syncthreads();
   if (warp == 0) {
-    const int ni = wl < nw ? packs[wl].n : 0, ki = wl < nw ? packs[wl].n_run : 0;
-    const int nn = warp_inclusive(ni), kk = warp_inclusive(ki);
+    const int ki = wl < nw ? packs[wl].n_run : 0;
+    const int kk = warp_inclusive(ki);
     int b = 0;
-    if (wl == 31 && nn) b = atomicAdd(&d.ctl->n_tl[t & 1], nn);
-    const int tl0 = __shfl_sync(0xffffffffu, b, 31);
-    if (wl == 31 && kk) b = atomicAdd(&d.ctl->n_run[t & 1], kk);
+    if (wl == 31 && kk) b = atomicAdd(&d.ctl->pk_run, kk);
     const int run0 = __shfl_sync(0xffffffffu, b, 31);
-    if (wl < nw) {
-      packs[wl].tl0 = tl0 + nn - ni;
-      packs[wl].run0 = run0 + kk - ki;
-    }
+    if (wl < nw) packs[wl].run0 = run0 + kk - ki;
   }
   __syncthreads();
 #pragma unroll 1
-  for (int i = wl; i < n; i += 32) d.tl[P.tl0 + i] = P.slot[i];
-#pragma unroll 1
-  for (int q = wl; q < k; q += 32) d.runs[P.run0 + q] = make_int2(P.tl0 + P.first[q], P.first[q + 1] - P.first[q]);
+  for (int q = 0; q < k; q++) {
+    const int i = P.first[q] + wl;
+    d.tl[(size_t)(P.run0 + q) * 32 + wl] = i < P.first[q + 1] ? P.slot[i] : -1;
+  }
   __syncthreads();
 }
 
-// One thread per lane slot settles the lane's front; level by level the loads are: slot
-// arrays, front record and link record, rear record of the next lane.  The runs of the move
-// phase are packed by the last blocks of the grid, which have fewer slots.
+// The whole packing of step t, by all blocks.
+__device__ __forceinline__ void seg_pack_all(const SegDev& d, SegPack* packs, int t) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) d.ctl->pk_step = t + 1;
+  // about one run per resident warp when there are few vehicles
+  const int most = max(32, min(kRunVeh, max(d.ctl->nact[(t + 1) & 1], d.ctl->pk_veh) / d.packed));
+  const int step = (int)(blockDim.x >> 5) * kPackSlots;
+#pragma unroll 1
+  for (int k = blockIdx.x; k * step < d.n_slots; k += gridDim.x) seg_pack(d, packs, k * step, most, t);
+}
+
+// One thread per lane (packed: of the listed links) settles the lane's front; level by level
+// the loads are: slot arrays, front record and link record, rear record of the next lane.
 template <bool TYPES, bool TAPE>
-__device__ __forceinline__ void seg_front(const SegDev& d, SegPack* packs, int t) {
+__device__ __forceinline__ void seg_front(const SegDev& d, int t) {
   const RearRec* rin = d.rear2 + (size_t)(t & 1) * d.n_slots;
   const unsigned tag = (unsigned)t + 1u;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const int next = (t + 1) & 1;
-    d.ctl->tm = t;
-    d.ctl->nact[t & 1] = 0;
-    d.ctl->n_bigl[next] = d.ctl->n_tl[next] = d.ctl->n_run[next] = d.ctl->n_late[next] = 0;
-  }
+  int n = d.n_slots, pk = 0;
   if (d.packed) {
-    // about one run per resident warp when there are few vehicles
-    const int most = max(32, min(kRunVeh, d.ctl->nact[(t + 1) & 1] / d.packed));
-    const int step = (int)(blockDim.x >> 5) * kPackSlots;
-#pragma unroll 1
-    for (int k = (int)(gridDim.x - 1 - blockIdx.x); k * step < d.n_slots; k += gridDim.x)
-      seg_pack(d, packs, k * step, most, t);
+    const int p = (t + 1) & 1;
+    const Ctl* c = d.ctl;
+    pk = c->pk_step;
+    n = 32 * (pk == t + 1 ? c->pk_run : c->n_run[p] + c->add_run[p]);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const int q = t & 1, p = q ^ 1;
+    Ctl* c = d.ctl;
+    c->tm = t;
+    c->nact[q] = 0;
+    c->n_run[q] = n >> 5;
+    c->add_run[q] = 0;
+    c->n_bigl[p] = c->n_late[p] = 0;
   }
   const int wl = threadIdx.x & 31;
 #pragma unroll 1
-  GRID_STRIDE(g, d.n_slots) {
+  GRID_STRIDE(k, n) {
+    const int g = d.packed ? d.tl[k] : k;
+    if (g < 0) continue;
     const uint32_t r = d.rng[g];
-    const int cnt = (int)(r >> 16), end = (int)(r & 0xffffu) + cnt;
-    // (few groups: the slot's other arrays are loaded along with its range; many: only for
-    // the slots with vehicles)
+    const int cnt = rng_count(r), end = rng_start(r) + cnt;
+    // (the slot's other arrays are loaded along with its range)
     const float4* ls = reinterpret_cast<const float4*>(d.lstat + g);
-    uint32_t info = 0;
-    int2 sg = make_int2(0, 0);
-    float4 A, B;
-    if (!d.packed || cnt) {
-      info = d.sinfo[g];
-      sg = d.lane_seg[g];
-      B = ls[1];
-      A = ls[0];
-    }
+    const uint32_t info = d.sinfo[g];
+    const int2 sg = d.lane_seg[g];
+    const float4 B = ls[1], A = ls[0];
     const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1, ctrl = ctrl_of(info);
-    if (!d.packed) {
+    if (d.packed) {
+      if (lane == lanes - 1 && end > 0) seg_check_link(d, g, lanes, end, sg.y, t);
+    } else {
       const int total = __shfl_sync(0xffffffffu, end, (wl + lanes - 1 - lane) & 31);
-      const bool big = total > 0 && seg_check_link(d, g, lane, lanes, total, sg.y, t);
+      if (lane == lanes - 1 && total > 0) seg_check_link(d, g, lanes, total, sg.y, t);
+      const bool big = seg_big(total, lanes);
       // parts of about the same number of vehicles, 16 at least
       const int w = big ? 0 : cnt, all = __reduce_add_sync(0xffffffffu, w);
       unsigned long long cuts = ~0ull;
@@ -380,10 +392,8 @@ __device__ __forceinline__ void seg_front(const SegDev& d, SegPack* packs, int t
     if (f.nxt >= 0 && !closed && xo >= A.x && (!lead || (xo - A.x) <= room)) {
       fl |= kSegCand;
       atomicMin(&d.best2[gt], seg_key(t, seg_rr(info, t), lane, (int)(info >> 16 & 255u)));
-      // a link with nothing else to do is listed for the vehicle that may enter it
-      const int gl = f.nlb >> 3;
-      const uint32_t rl = d.packed ? d.rng[gl + (f.nlb & 7)] : 1u;
-      if ((rl & 0xffffu) + (rl >> 16) == 0 && d.qnext[gl] > t && atomicExch(&d.claim[f.nxt], t + 1) != t + 1)
+      // an unlisted link is noted for the vehicle that may enter it
+      if (d.packed && d.listed[f.nxt] != pk && atomicExch(&d.listed[f.nxt], pk) != pk)
         d.late[atomicAdd(&d.ctl->n_late[t & 1], 1)] = f.nxt;
       // the record after crossing, pulled by the target lane if this bid wins (a bidding
       // front never changes lanes: its own-lane move reaches the link end)
@@ -415,6 +425,7 @@ struct SegLane {
   bool on;               // part of the run
   bool ext;              // a crossing vehicle comes in (its record: cr2[src])
   bool due;              // first lane of a link whose departure queue is due
+  bool done;             // a whole block has written the lane in this step
   int g, to, src, cnt, start, seg;
   int2 fr;
   float4 la, lb;
@@ -657,6 +668,17 @@ __device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& l
   };
   const RearRec* rin = d.rear2 + (size_t)(t & 1) * d.n_slots;
   const unsigned tag = (unsigned)t + 1u;
+  auto stage = [&](int i, int j, const VehRec& r) {
+    S.x[i] = r.x;
+    S.v[i] = r.v;
+    S.vid[i] = r.vid;
+    S.nxt[i] = r.nxt;
+    S.nlb[i] = r.nlb;
+    S.ri[i] = r.ri;
+    S.tau[i] = r.tau;
+    S.meta[i] = r.meta >> 3 & ~12u;
+    S.jo[i] = (uint8_t)j;
+  };
   // ---- lane tables, crossing vehicles
   int n = 0, my_pos = 0;
   const bool on = ln.on, due = ln.on && ln.due;
@@ -693,33 +715,13 @@ __device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& l
     }
     if (ln.on && ln.ext) {
       const int i = n + __popc(xm & lt);
-      const VehRec r = seg_load(d.cr2 + ln.src);
-      S.x[i] = r.x;
-      S.v[i] = r.v;
-      S.vid[i] = r.vid;
-      S.nxt[i] = r.nxt;
-      S.nlb[i] = r.nlb;
-      S.ri[i] = r.ri;
-      S.tau[i] = r.tau;
-      S.meta[i] = r.meta >> 3 & ~12u;
-      S.jo[i] = kNew;
+      stage(i, kNew, seg_load(d.cr2 + ln.src));
       S.it[i] = (uint8_t)tid;
     }
   }
   sync();
   if (NT != 32) n = S.n;
   // ---- vehicles
-  auto stage = [&](int i, int j, const VehRec& r) {
-    S.x[i] = r.x;
-    S.v[i] = r.v;
-    S.vid[i] = r.vid;
-    S.nxt[i] = r.nxt;
-    S.nlb[i] = r.nlb;
-    S.ri[i] = r.ri;
-    S.tau[i] = r.tau;
-    S.meta[i] = r.meta >> 3 & ~12u;
-    S.jo[i] = (uint8_t)j;
-  };
   if (NT == 32) {
     // two windows of 32 vehicles at a time, so that their loads overlap
 #pragma unroll 1
@@ -959,7 +961,7 @@ __device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& l
       const int s = inc - cnt - first;
       S.wb[tid] = S.sg[tid] + s;
       S.cn[tid] = cnt;
-      d.rng[S.gs[tid]] = (uint32_t)s | (uint32_t)cnt << 16;
+      d.rng[S.gs[tid]] = (uint32_t)s | (uint32_t)cnt << 16 | (NT == 32 ? 0u : 2u + (unsigned)(t & 1)) << 30;
     }
   }
   // a stayer not below the next stayer of its lane: the whole lane is ranked by counting
@@ -1044,7 +1046,7 @@ __device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& l
 // What the thread of slot g needs (g < 0: none).
 __device__ __forceinline__ SegLane seg_lane(const SegDev& d, int g, int t) {
   SegLane ln;
-  ln.on = ln.ext = ln.due = false;
+  ln.on = ln.ext = ln.due = ln.done = false;
   ln.g = g;
   ln.to = ln.src = ln.cnt = ln.start = ln.seg = 0;
   ln.fr = make_int2(0, 0);
@@ -1062,8 +1064,9 @@ __device__ __forceinline__ SegLane seg_lane(const SegDev& d, int g, int t) {
   ln.seg = d.lane_seg[g].x;
   ln.to = d.slot_to[g];
   ln.fr = d.fres[g];
-  ln.start = (int)(r & 0xffffu);
-  ln.cnt = (int)(r >> 16);
+  ln.start = rng_start(r);
+  ln.cnt = rng_count(r);
+  ln.done = (r >> 30) == 2u + (unsigned)(t & 1);
   const unsigned info = __float_as_uint(ln.lb.z);
   if (ln.cnt == 0) ln.fr.y = 0;   // an empty lane's record is an older step's
   if (epoch_current(bk, t)) {
@@ -1080,8 +1083,8 @@ __device__ __forceinline__ SegLane seg_lane(const SegDev& d, int g, int t) {
   return ln;
 }
 
-// A link without vehicles or departures that crossing vehicles may have entered, by one
-// thread: at most one vehicle per lane, already in order.
+// An unlisted link (no vehicles, no departures) that crossing vehicles may have entered, by
+// one thread: at most one vehicle per lane, already in order.
 __device__ __forceinline__ void seg_enter(const SegDev& d, int e, int t) {
   const int g0 = d.lslot[e];
   const int seg = d.lane_seg[g0].x, tail = d.stail[g0], to = d.slot_to[g0];
@@ -1104,9 +1107,39 @@ __device__ __forceinline__ void seg_enter(const SegDev& d, int e, int t) {
   }
 }
 
+// The links noted in this step, 32 per warp: their vehicles, and their place in the lists of
+// the steps until the next packing.
+__device__ __forceinline__ void seg_late(const SegDev& d, int first, int t) {
+  const int wl = threadIdx.x & 31, q = t & 1;
+  const bool in = first + wl < d.ctl->n_late[q];
+  int lanes = 0, g0 = 0;
+  if (in) {
+    const int e = d.late[first + wl];
+    g0 = d.lslot[e];
+    lanes = (int)(d.sinfo[g0] >> 3 & 7u) + 1;
+    seg_enter(d, e, t);
+  }
+  const int inc = warp_inclusive(lanes);
+  const int n = __popc(__ballot_sync(0xffffffffu, in));
+#pragma unroll 1
+  for (int s = 0, before = 0; s < n;) {
+    const int e = s + __popc(__ballot_sync(0xffffffffu, in && wl >= s && inc - before <= 32)) - 1;
+    const int to = __shfl_sync(0xffffffffu, inc, e);
+    int run = 0;
+    if (wl == 0) run = d.ctl->n_run[q] + atomicAdd(&d.ctl->add_run[q], 1);
+    int32_t* row = d.tl + (size_t)__shfl_sync(0xffffffffu, run, 0) * 32;
+    if (wl >= to - before) row[wl] = -1;
+    if (wl >= s && wl <= e)
+#pragma unroll 1
+      for (int l = 0; l < lanes; l++) row[inc - lanes - before + l] = g0 + l;
+    before = to;
+    s = e + 1;
+  }
+}
+
 // The move phase of step t.  First the links left to whole blocks, then the runs, one per
 // warp (one whose incoming vehicles take it beyond the staging area in several passes), then
-// the empty links that vehicles enter, 32 per warp.  Units of one run per warp are dealt to
+// the unlisted links that vehicles enter, 32 per warp.  Units of one run per warp are dealt to
 // the blocks after the big links (a unit each); few runs spread over all blocks.
 template <bool OUT, bool TYPES, bool TAPE>
 __device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, int t) {
@@ -1124,22 +1157,21 @@ __device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, i
   }
   SegSmem& S = *reinterpret_cast<SegSmem*>(smem + (size_t)warp * kSegWarpBytes);
   const int n_grp = d.n_slots >> 5;
-  const int n_run = d.packed ? d.ctl->n_run[t & 1] : n_grp * d.parts, n_late = d.ctl->n_late[t & 1];
+  const int n_run = d.packed ? d.ctl->n_run[t & 1] : n_grp * d.parts;
+  const int n_late = d.packed ? d.ctl->n_late[t & 1] : 0;
   const int n_all = n_run + (n_late + 31) / 32;
   const int per = min((int)(blockDim.x >> 5), (n_all + (int)gridDim.x - 1) / (int)gridDim.x);
   const int b0 = (int)((blockIdx.x + gridDim.x - (unsigned)nbig % gridDim.x) % gridDim.x);
 #pragma unroll 1
   for (int k = b0 * per + warp; warp < per && k < n_all; k += gridDim.x * per) {
     if (k >= n_run) {
-      const int i = (k - n_run) * 32 + wl;
-      if (i < n_late) seg_enter(d, d.late[i], t);
+      seg_late(d, (k - n_run) * 32, t);
       continue;
     }
     int g, ja = 0, jend;
     if (d.packed) {
-      const int2 run = d.runs[k];
-      jend = run.y;
-      g = wl < jend ? d.tl[run.x + wl] : -1;
+      g = d.tl[(size_t)k * 32 + wl];
+      jend = __popc(__ballot_sync(0xffffffffu, g >= 0));
     } else {   // part p of group k - p n_grp
       const int p = k / n_grp, grp = k - p * n_grp;
       const unsigned long long cuts = d.cuts[grp];
@@ -1151,11 +1183,13 @@ __device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, i
 #pragma unroll 1
     do {
       SegLane ln = seg_lane(d, g, t);
-      if (!d.packed) {   // empty slots, links left to whole blocks
+      {   // not: empty slots, links left to whole blocks (one may have been through, and have
+          // left fewer vehicles: its last lane's range, one word, tells either way)
         const unsigned info = __float_as_uint(ln.lb.z);
-        if (ctrl_of(info) == kCtrlPad) ln.on = false;
         const int lane = (int)(info & 7u), lanes = (int)(info >> 3 & 7u) + 1;
-        if (seg_big(__shfl_sync(0xffffffffu, ln.start + ln.cnt, (wl + lanes - 1 - lane) & 31), lanes)) ln.on = false;
+        const bool big = __shfl_sync(0xffffffffu, ln.done || seg_big(ln.start + ln.cnt, lanes) ? 1 : 0,
+                                     (wl + lanes - 1 - lane) & 31) != 0;
+        if (ctrl_of(info) == kCtrlPad || big) ln.on = false;
       }
       ln.on = ln.on && wl >= ja && wl < jend;
       const int w = ln.on ? ln.cnt + (ln.ext ? 1 : 0) + (ln.due ? 1 : 0) : 0;
@@ -1181,7 +1215,10 @@ __device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, i
     if (s_cn[1]) atomicAdd(&c->lc_evals, (unsigned long long)s_cn[1]);
     if (s_cn[2]) atomicAdd(&c->arrived, (unsigned long long)s_cn[2]);
     if (s_cn[3]) atomicAdd(&c->departed, (unsigned long long)s_cn[3]);
-    if (blockIdx.x == 0) c->t = (long long)t + 1;
+    if (blockIdx.x == 0) {
+      c->t = (long long)t + 1;
+      c->pk_run = c->pk_veh = 0;   // for the next packing
+    }
   }
 }
 

@@ -87,6 +87,52 @@ def test_loop_routes_bitexact(G, lanes):
     run_lockstep(g, o, 400, 100)
 
 
+# more groups of lanes than resident warps: packed lists kept for several steps.  Chunks of 1, 7,
+# 8, 9 and more steps begin and end at every age of the lists; walks enter links that are not
+# in them, trips depart up to step 200, one link is left to a whole block.
+@pytest.mark.parametrize("n,lanes,mode", [(128, 2, 0), (104, 3, 0), (128, 2, 1)])
+def test_packed_lists_bitexact(G, n, lanes, mode):
+    import oracle
+    sc = _crowd(_grid(n=n, lanes=lanes, n_trips=5000, loop=mode == 1), 77, 120)
+    sc["params"]["loop_routes"] = 0
+    sc["init_state"] = _state(sc, 77, 47, 4.2)
+    g, o = setup_pair(sc, G.Sim, oracle.OracleSim)
+    if mode:
+        g.set_exec(mode=1, threads=256, blocks_per_sm=2)
+    for total, chunk in [(3, 1), (14, 7), (8, 8), (18, 9), (21, 21), (100, 50), (130, 130)]:
+        run_lockstep(g, o, total, chunk)
+    assert o.counters()["arrived"] > 20
+
+
+# a dense network, several runs per warp, with links that hold as many vehicles as a whole block
+# is set to, or a few more, and lose some: no second warp may take them in the same step
+@pytest.mark.parametrize("mode", [0, 1])
+def test_links_about_the_staging_area_bitexact(G, mode):
+    import oracle
+    sc = S.small_grid(n=128, n_trips=580000, lanes=3, seed=S.BASE_SEED + 6, window_steps=200)
+    net = sc["network"]
+    lf, lt = net["link_from"].astype(np.int64), net["link_to"].astype(np.int64)
+    n_links, n = len(lf), sc["demand"]["n_trips"]
+    out = np.argsort(lf, kind="stable")
+    k = np.searchsorted(lf[out], lt)
+    nxt = np.where(lt[out[k]] == lf, out[np.minimum(k + 1, n_links - 1)], out[k])   # not back
+    crowded = np.arange(50, n_links, 97)
+    many = 93 + np.arange(len(crowded)) % 4
+    at = np.concatenate([np.repeat(crowded, many), np.tile(np.setdiff1d(np.arange(n_links), crowded), 9)])[:n]
+    sc["routes"] = dict(offsets=3 * np.arange(n + 1, dtype=np.int32),
+                        links=np.stack([at, nxt[at], nxt[nxt[at]]], 1).reshape(-1).astype(np.int32))
+    order = np.argsort(at, kind="stable")
+    rank = np.empty(n, np.int64)
+    rank[order] = np.arange(n) - np.searchsorted(at[order], at[order])
+    x = 199.0 - 6.0 * (rank // 3)
+    sc["init_state"] = dict(status=np.ones(n, np.uint8), link=at.astype(np.int32), lane=(rank % 3).astype(np.int32),
+                            cursor=np.zeros(n, np.int32), x=x.astype(np.float32), v=np.full(n, 9.0, np.float32))
+    g, o = setup_pair(sc, G.Sim, oracle.OracleSim)
+    if mode:
+        g.set_exec(mode=1, threads=256, blocks_per_sm=1)
+    run_lockstep(g, o, 12, 4)
+
+
 # vehicles per lane of a 200 m link: up to a warp's staging area, past it, past the link's
 # segment (84 + 2 vehicles), past a block's staging area
 @pytest.mark.parametrize("per_lane,spacing", [(40, 5.0), (46, 4.3), (47, 4.2), (120, 1.5), (560, 0.3), (60, 0.0)])
