@@ -111,7 +111,8 @@ __device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, in
     }
     seg_front<TYPES, false>(d, t);
     if (!grid_barrier(gs, err, limit)) return;
-    if (*(volatile int*)&d.ctl->grow) return;   // set before the barrier, the same for every block
+    // set before the barrier, the same for every block (one thread asks: see step_timed_out)
+    if (__syncthreads_or(threadIdx.x == 0 && *(volatile int*)&d.ctl->grow)) return;
     seg_move<OUT, TYPES, false>(d, smem, t);
     if (!grid_barrier(gs, err, limit)) return;
   }

@@ -88,7 +88,8 @@ __device__ __forceinline__ int rng_start(uint32_t r) { return (int)(r & 0xffffu)
 __device__ __forceinline__ int rng_count(uint32_t r) { return (int)(r >> 16 & 0x3fffu); }
 
 __device__ __forceinline__ bool seg_stopped(const SegDev& d) {
-  return (*(volatile int*)&d.ctl->err & kErrTimeout) != 0 || *(volatile int*)&d.ctl->grow != 0;
+  const int err = d.ctl->err, grow = d.ctl->grow;   // (cached: see step_timed_out)
+  return (err & kErrTimeout) != 0 || grow != 0;
 }
 
 __device__ __forceinline__ VehRec seg_load(const VehRec* p) {

@@ -38,9 +38,10 @@ __device__ __forceinline__ int count_in_lane(const Dev& d, int g) {
 // A step kernel returns at entry once a bounded wait of this step (or of an earlier
 // one) ran out: the state is then undefined, the host reports SIM_ETIMEOUT and refuses
 // to step until the state is reset, and no kernel works on partly computed scratch.
-__device__ __forceinline__ bool step_timed_out(const Dev& d) {
-  return (*(volatile int*)&d.ctl->err & kErrTimeout) != 0;
-}
+// A plain load, after the wait for the kernels before: as a volatile one it took 0.6 to 1.3 us
+// of every kernel (ring of 50 vehicles, 7 kernels a step: 31 -> 22 us; 1,000 queues of 570
+// vehicles: 121 -> 111 us a step).
+__device__ __forceinline__ bool step_timed_out(const Dev& d) { return (d.ctl->err & kErrTimeout) != 0; }
 
 __device__ __forceinline__ bool is_holder(const Dev& d, const LinkRec& L, int t, int vid, int lane,
                                           bool front) {
@@ -183,8 +184,8 @@ __device__ __forceinline__ bool grid_barrier(GridSync* gs, int* err, long long l
       atomicAdd(&gs->gen, 1u);
     } else {
       const long long t0 = clock64();
-      while (*vgen == g) {
-        if ((*verr & kErrTimeout) || clock64() - t0 > limit) {
+      for (unsigned spin = 1; *vgen == g; spin++) {   // (few looks at the error word: it is every block's)
+        if ((spin % 64 == 0 && (*verr & kErrTimeout)) || clock64() - t0 > limit) {
           atomicOr(err, kErrTimeout);
           ok = 0;
           break;
