@@ -633,7 +633,9 @@ def run_cuda(args):
     achieved_fl = STEP_KERNEL_BYTES * avg_active_fl / (step_ms_fl * 1e-3) / 1e9
     achieved = STEP_KERNEL_BYTES * avg_active / (step_ms * 1e-3) / 1e9
     whole = WHOLE_STEP_BYTES * (veh_steps / args.steps) / (ms / args.steps * 1e-3) / 1e9
-    impl_gbs = {k: IMPL_BYTES[k] * avg_active / (kms[k] / args.steps * 1e-3) / 1e9 for k in IMPL_BYTES if k in kms}
+    # (the bytes are the sorted form's; in link segments its other kernels take no time)
+    impl_gbs = {k: IMPL_BYTES[k] * avg_active / (kms[k] / args.steps * 1e-3) / 1e9
+                for k in IMPL_BYTES if k in kms and kms.get("scatter")}
 
     # -- end to end through the C ABI with host buffers: load the snapshot from pinned host
     #    memory, then every step read positions and speeds back to pinned host memory.  The
