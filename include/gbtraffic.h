@@ -189,15 +189,17 @@ int sim_step_timed(sim_handle* h, int32_t n_steps, float* kernel_ms);
 const char* sim_kernel_name(int32_t k);
 
 /* Kernel launches sim_step has made on this handle since its creation, into *launches:
- * in graph execution the kernels of the captured step graph, per step; in persistent
- * execution one cooperative launch per sim_step call.  (Launches of the other calls
+ * in graph execution the kernels of the captured step graphs (networks of 2,048 lanes
+ * and more 2 per step and now and then a packing of their busy links, smaller ones 7 to
+ * 9); in persistent execution one cooperative launch per sim_step call.  (Launches of the other calls
  * are not counted.)  Errors: SIM_EINVAL on a NULL argument. */
 int sim_launch_count(sim_handle* h, int64_t* launches);
 
-/* How sim_step runs the steps.  SIM_EXEC_GRAPH: one CUDA graph of the step's kernels
- * per step, grid = grid_per_sm x SMs blocks of 256 threads for the kernels that do not
- * size their own grid (the chunk kernel runs one resident wave); the chunk kernel's
- * waits for its staged chunks (bulk copies into shared memory) are bounded by
+/* How sim_step runs the steps.  SIM_EXEC_GRAPH: CUDA graphs of one or eight steps,
+ * grid = grid_per_sm x SMs blocks of 256 threads for the kernels that do not size their
+ * own grid.  Networks below 2,048 lanes, and those whose links are mostly longer than a
+ * staged chunk holds, run the sorted form of the step: its chunk kernel's
+ * waits for staged chunks (bulk copies into shared memory) are bounded by
  * barrier_timeout_cycles SM cycles (<= 0: 2e9), after which sim_step returns
  * SIM_ETIMEOUT (the state is then undefined until the next sim_write_state /
  * sim_route, and stepping calls return SIM_ESTATE until then).  SIM_EXEC_PERSISTENT: all
@@ -475,8 +477,8 @@ int sim_sssp_static(int32_t n_nodes, int32_t n_links, const int32_t* out_start, 
 /* Test hook of sim_sssp_static (no counterpart in the paper): sets the two counters the
  * fixed array keeps across calls, the search epoch that tags distance words and the
  * round number that tags queue flags.  After any call that leaves either at 2^30 or
- * more, sim_sssp_static puts the array back to its first-use state (distance words
- * all-ones, flags and counters zero) so that neither counter can wrap around in a
+ * more, sim_sssp_static puts the array back to its first-use state (node records
+ * all-ones, counters zero) so that neither counter can wrap around in a
  * long-lived process; this hook lets a test reach that point without a billion calls.
  * The counters may only be moved forward (below their current values, stale tags in
  * the array would look current).  Same set-up and serialisation rules as

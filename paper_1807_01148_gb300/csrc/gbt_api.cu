@@ -252,12 +252,13 @@ int upload(sim_handle* h, T** p, const T* src, size_t n) {
 // Which form the steps run in.  Graph execution: networks of kSegLanes lanes and more in the
 // segments, smaller ones in the sorted form, whose launches per step (7 to 9) sim_launch_count
 // reports for small networks and callers rely on there.  Persistent execution (one launch
-// either way): the segments on any network.  Measured, us per step, sorted -> segments: 20 x
-// 20 grid (3,040 lanes, 2,050 vehicles) 41.6 -> 22.2; town of 6,700 lanes 16.3 -> 8.6 (with its
-// share of planning); district of 42,000 lanes with outputs and trucks 78 -> 71.
-// On networks with more groups of lanes than resident warps of the move phase, in packed
-// lists (SegDev::packed; us per step): 64 copies of a grid 76.8 -> 64.5; metro, 782,000 lanes,
-// 2.11M vehicles 274 -> 269 and, in the persistent launch with 500,000, 89 -> 78.
+// either way): the segments on any network.  Measured, us per step with the reads of the state,
+// sorted -> segments: 20 x 20 grid (3,040 lanes, 2,050 vehicles) 43.0 -> 18.5; town of 6,700
+// lanes (with its share of planning) 60.9 -> 28.4; district of 42,000 lanes with outputs and
+// trucks 94.6 -> 86.5.  On networks with more groups of lanes than resident warps of the move
+// phase, in packed lists (SegDev::packed): 64 copies of a grid (321,000 lanes) 76.6 -> 62.2;
+// metro (782,000 lanes) with 2.11M vehicles 273 -> 267 and, in the persistent launch, with
+// 173,000 90 -> 76.
 // Not in the segments: networks where links longer than a staged chunk carry most of the
 // road, for which the sorted form has its big-chunk kernel (1,000 queues of 570 vehicles: 118
 // against 122).
@@ -1411,9 +1412,7 @@ int enqueue_graph_steps(sim_handle* h, int n, bool tape, bool count) {
   if (dirty || form != h->seg) {
     g1.drop();
     g8.drop();
-    if (!tape) {
-      h->samp1.drop();
-    }
+    if (!tape) h->samp1.drop();
     steps = 0;
     dirty = false;
     form = h->seg;
