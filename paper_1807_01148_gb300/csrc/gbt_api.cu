@@ -388,6 +388,13 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   return SIM_OK;
 }
 
+// Buffer A -> the segments that are there.  The import empties the packed lists, so the next
+// step has to pack them whatever their age was.
+cudaError_t seg_import(sim_handle* h) {
+  h->pack_age = 1 << 20;
+  return launch_seg_import(h->d, h->grid, h->stream);
+}
+
 // Buffer A -> segments.  When they cannot hold the state (memory, a link with more vehicles
 // than a block stages) the sorted form goes on: h->seg stays false, h->seg_off is set, and
 // the call succeeds.
@@ -400,7 +407,7 @@ int seg_from_sorted(sim_handle* h) {
       h->seg_off = true;
       break;
     }
-    cudaError_t e = launch_seg_import(h->d, h->grid, h->stream);
+    cudaError_t e = seg_import(h);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&h->mirror->c, h->d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -408,7 +415,6 @@ int seg_from_sorted(sim_handle* h) {
     const int grow = h->mirror->c.grow;
     if (!grow) {
       h->seg = true;
-      h->pack_age = 1 << 20;
       return SIM_OK;
     }
     if (grow == 2 || attempt == 1) {
@@ -2057,7 +2063,7 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
   for (int sg = nseg - 1; sg >= 0 && e == cudaSuccess && rc == SIM_OK; sg--) {
     const int j0 = sg * seg, j1 = std::min(n_steps, (sg + 1) * seg);
     e = ckpt_copy(h, ck + (size_t)sg * CL.bytes, false);
-    if (e == cudaSuccess && replay_seg) e = launch_seg_import(h->d, h->grid, h->stream);   // fits: the forward pass did
+    if (e == cudaSuccess && replay_seg) e = seg_import(h);   // fits: the forward pass did
     if (e == cudaSuccess) e = cudaMemsetAsync(h->tape, 0, (size_t)seg * nt * sizeof(TapeRec), h->stream);
     launch_tape_begin(h->d, h->stream);
     h->seg = replay_seg;
