@@ -1,0 +1,66 @@
+"""Links in segments whose vehicles come and go all at once, bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+from paper_1807_01148_gb300 import scenarios as S
+
+from .parity import run_lockstep, setup_pair
+from .test_seg_gpu import _grid
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_1807_01148_gb300 import gbtraffic
+    return gbtraffic
+
+
+def emptied_link(n, second):
+    """100 vehicles at the end of their last link (more than a warp stages) and one that comes
+    two steps later: a departure, or a vehicle that crosses into the link.  Nothing else is on
+    the road, so nobody works on the link in between."""
+    sc = _grid(n=n, n_trips=101)
+    net = sc["network"]
+    lf, lt = net["link_from"].astype(np.int64), net["link_to"].astype(np.int64)
+    # a link and one before it, straight on, in another group of 32 lanes (2 lanes each)
+    L, F, out = next((b, a, c) for b in range(40, len(lf)) for a in np.flatnonzero(lt == lf[b])
+                     if lt[b] - lf[b] == lt[a] - lf[a] and a // 16 != b // 16
+                     for c in np.flatnonzero(lf == lt[b])[:1] if lt[c] != lf[b])
+    if second == "departs":
+        legs = [[L]] * 100 + [[L, out]]
+    else:
+        legs = [[L]] * 100 + [[F, L, out]]
+    sc["routes"] = dict(offsets=np.r_[0, np.cumsum([len(q) for q in legs])].astype(np.int32),
+                        links=np.concatenate(legs).astype(np.int32))
+    sc["demand"]["depart_step"][:] = 0
+    sc["demand"]["depart_step"][100] = 2
+    k = np.arange(101)
+    st = dict(status=np.ones(101, np.uint8), link=np.full(101, L, np.int32), lane=(k % 2).astype(np.int32),
+              cursor=np.zeros(101, np.int32), x=np.full(101, net["link_length_m"][L], np.float32),
+              v=np.full(101, 9.0, np.float32))
+    if second == "departs":
+        st["status"][100] = st["link"][100] = st["x"][100] = st["v"][100] = 0
+    else:
+        st["link"][100], st["x"][100] = F, net["link_length_m"][F] - 13.0
+    st["lane"][100] = 0
+    sc["init_state"] = st
+    return sc, L
+
+
+@pytest.mark.parametrize("n", [24, 160], ids=["parts", "packed"])
+@pytest.mark.parametrize("second", ["departs", "crosses"])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_link_emptied_by_a_block_bitexact(G, n, second, mode):
+    import oracle
+    sc, L = emptied_link(n, second)
+    g, o = setup_pair(sc, G.Sim, oracle.OracleSim)
+    if mode:
+        g.set_exec(mode=1, threads=256, blocks_per_sm=1)
+    run_lockstep(g, o, 1, 1)
+    assert o.counters()["arrived"] == 100   # the link is empty
+    run_lockstep(g, o, 1, 1)
+    assert not (o.state()["link"][o.state()["status"] == 1] == L).any()
+    run_lockstep(g, o, 1, 1)
+    assert (o.state()["link"][o.state()["status"] == 1] == L).sum() == 1   # comes in the third step
+    run_lockstep(g, o, 20, 5)
