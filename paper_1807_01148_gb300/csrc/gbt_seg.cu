@@ -55,7 +55,8 @@ __global__ void __launch_bounds__(kSegThreads, 3) k_seg_move(SegDev d) {
 }
 
 // Sec. 6.4 per-edge sample of the state at step t (see ph_edge_sample): one thread per link
-// over its segment.
+// over its segment.  After the front phase, which may stop the step (Ctl::grow): a step that
+// does not take place now is sampled when it does.
 __device__ __forceinline__ void seg_edge_sample(const SegDev& d, long long t) {
   if (t % d.samp_every != 0) return;
   const long long k = t / d.samp_every;
@@ -96,7 +97,8 @@ __global__ void k_seg_edge_sample(SegDev d) {
 }
 
 // ------------------------------------------------------------------ persistent step
-// All steps in one cooperative launch: two grid barriers per step.
+// All steps in one cooperative launch: two grid barriers per step, and one more where the lists
+// are packed or the links sampled.
 template <bool OUT, bool TYPES>
 __device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, int n_steps, long long limit,
                                                unsigned char* smem) {
@@ -104,7 +106,6 @@ __device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, in
   const int t0 = (int)*(volatile long long*)&d.ctl->t;
   for (int step = 0; step < n_steps; step++) {
     const int t = t0 + step;
-    if (d.acc_u) seg_edge_sample(d, t);
     if (d.packed && step % kPackSteps == 0) {
       seg_pack_all(d, reinterpret_cast<SegPack*>(smem), t);
       if (!grid_barrier(gs, err, limit)) return;
@@ -113,6 +114,10 @@ __device__ __forceinline__ void seg_persistent(const SegDev& d, GridSync* gs, in
     if (!grid_barrier(gs, err, limit)) return;
     // set before the barrier, the same for every block (one thread asks: see step_timed_out)
     if (__syncthreads_or(threadIdx.x == 0 && *(volatile int*)&d.ctl->grow)) return;
+    if (d.acc_u && t % d.samp_every == 0) {   // the move phase changes what it reads
+      seg_edge_sample(d, t);
+      if (!grid_barrier(gs, err, limit)) return;
+    }
     seg_move<OUT, TYPES, false>(d, smem, t);
     if (!grid_barrier(gs, err, limit)) return;
   }
@@ -460,8 +465,8 @@ void launch_seg_pack(const SegDev& d, cudaStream_t s) {
 }
 
 void launch_seg_step(const SegDev& d, int grid, cudaStream_t s) {
-  if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
   launch_seg_front(d, s);
+  if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
   launch_seg_move(d, s);
 }
 
@@ -476,8 +481,8 @@ cudaError_t launch_seg_steps_timed(const SegDev& d, int grid, cudaStream_t s, in
   for (int it = 0; it < n && err == cudaSuccess; it++) {
     cudaEventRecord(ev[0], s);
     if (d.packed && it % kPackSteps == 0) launch_seg_pack(d, s);
-    if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
     launch_seg_front(d, s);
+    if (d.acc_u) launch_pdl3(k_seg_edge_sample, grid, 256, 0, s, d);
     cudaEventRecord(ev[1], s);
     launch_seg_move(d, s);
     cudaEventRecord(ev[2], s);

@@ -4,7 +4,8 @@ import pytest
 
 from paper_1807_01148_gb300 import scenarios as S
 
-from .parity import run_lockstep, setup_pair
+from .parity import compare, run_lockstep, setup_pair
+from .test_outputs_gpu import compare_outputs
 from .test_seg_gpu import _grid
 
 pytestmark = pytest.mark.gpu
@@ -64,3 +65,49 @@ def test_link_emptied_by_a_block_bitexact(G, n, second, mode):
     run_lockstep(g, o, 1, 1)
     assert (o.state()["link"][o.state()["status"] == 1] == L).sum() == 1   # comes in the third step
     run_lockstep(g, o, 20, 5)
+
+
+def filling_link(most, depart):
+    """A link that holds as many vehicles (overlapping) as its segment or a block's staging area
+    takes, and one more from step `depart` + 1 on."""
+    sc = _grid(n=24, n_trips=most + 1)
+    net = sc["network"]
+    lf, lt = net["link_from"].astype(np.int64), net["link_to"].astype(np.int64)
+    # an east-west link whose head stays green north-south for the first 12 steps
+    phase = -net["signal_offset_ds"] % net["signal_cycle_ds"]
+    red = (phase + 12 * 5 < net["signal_green_ds"])[lt]
+    ew = net["node_y_dm"][lf] == net["node_y_dm"][lt]
+    L = int(np.flatnonzero(red & ew)[5])
+    out = int(np.flatnonzero((lf == lt[L]) & (lt != lf[L]))[0])
+    n = most + 1
+    sc["routes"] = dict(offsets=2 * np.arange(n + 1, dtype=np.int32), links=np.tile([L, out], n).astype(np.int32))
+    sc["demand"]["depart_step"][:] = 0
+    sc["demand"]["depart_step"][most] = depart
+    k = np.arange(n)
+    st = dict(status=np.ones(n, np.uint8), link=np.full(n, L, np.int32), lane=(k % 2).astype(np.int32),
+              cursor=np.zeros(n, np.int32), x=(199.0 - 170.0 * (k // 2) / (most // 2)).astype(np.float32),
+              v=np.zeros(n, np.float32))
+    for q in ("status", "link", "lane", "x"):
+        st[q][most] = 0
+    sc["init_state"] = st
+    return sc, L
+
+
+# 200 m of 2 lanes hold 84 vehicles of 5 m and 2 more that a step may bring; a block stages 1,024
+@pytest.mark.parametrize("most", [84, 1022])
+@pytest.mark.parametrize("depart", [0, 1])
+@pytest.mark.parametrize("how", ["graph", "persistent", "timed"])
+def test_sample_of_a_step_that_did_not_fit(G, most, depart, how):
+    import oracle
+    sc, L = filling_link(most, depart)
+    g, o = setup_pair(sc, G.Sim, oracle.OracleSim)
+    for q in (g, o):
+        q.set_outputs(7, sample_every=1, per_window=3, max_windows=4)
+    if how == "persistent":
+        g.set_exec(mode=1, threads=256, blocks_per_sm=1)
+    o.step(depart + 1)
+    assert (o.state()["link"] == L).sum() == most + 1   # the next step does not fit
+    o.step(12 - depart - 1)
+    g.step_timed(12) if how == "timed" else g.step(12)
+    compare(g, o, "filled")
+    compare_outputs(g, o, 7, "filled")
