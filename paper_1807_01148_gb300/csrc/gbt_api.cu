@@ -1512,6 +1512,19 @@ int enqueue_steps(sim_handle* h, long long t0, int n_steps) {
   return SIM_OK;
 }
 
+// What the next n steps need beside themselves, made beforehand: the step counter, the form of
+// the state, the graphs (a later launch of the same step count needs nothing more).
+int ready_steps(sim_handle* h, int n) {
+  if (int rc = check_horizon(h, n)) return rc;
+  if (int rc = seg_choose(h)) return rc;
+  if (h->exec.mode == SIM_EXEC_PERSISTENT) return SIM_OK;
+  if (int rc = enqueue_graph_steps(h, 0, false, false)) return rc;   // drops outdated graphs
+  SegDev d = h->d;
+  d.acc_u = nullptr;
+  if (int rc = capture_steps(h, h->step1, d, 1)) return rc;
+  return n >= kUnroll ? capture_steps(h, h->step8, d, kUnroll) : SIM_OK;
+}
+
 // After steps that stopped because a segment was full (the step they stopped at has not
 // begun): back to the sorted form, larger segments or none.
 int seg_regrow(sim_handle* h, int grow) {
@@ -2187,6 +2200,9 @@ int sim_autotune(sim_handle* h, int32_t trial_steps, const char* cache_path, sim
     if ((rc = sim_step(h, trial_steps))) break;   // warm-up (builds the graphs of this step count)
     err = ckpt_copy(h, ck, false);
     if (err != cudaSuccess) break;
+    // the steps alone are timed: the restored state is in the sorted form, and graphs of eight
+    // steps are otherwise captured in the course of a run
+    if ((rc = ready_steps(h, trial_steps))) break;
     cudaEventRecord(e0, h->stream);
     if ((rc = sim_step(h, trial_steps))) break;
     cudaEventRecord(e1, h->stream);

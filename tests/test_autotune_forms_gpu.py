@@ -1,0 +1,22 @@
+"""The autotuner times steps alone (a restored state is brought into the form of the step, and
+graphs are captured, beforehand)."""
+import pytest
+
+from paper_1807_01148_gb300 import scenarios as S
+
+pytestmark = pytest.mark.gpu
+
+
+def _sim():
+    from paper_1807_01148_gb300 import gbtraffic as G
+    g = G.Sim(S.small_grid(n=6, n_trips=216, steps=600, window_steps=300))
+    g.route()
+    g.step(250)
+    return g
+
+
+def test_short_trials_pick_the_faster_form(tmp_path):
+    # 240 lanes: a step takes 21 us in graphs (sorted form), 14 us in the persistent launch
+    # (segments); laying the segments out takes some 60 us once
+    for k in range(3):
+        assert _sim().autotune(4, str(tmp_path / f"t{k}.jsonl"))["mode"] == 1
