@@ -2120,8 +2120,9 @@ std::string tune_key(const sim_handle* h) {
   mix((unsigned long long)h->nt);
   mix((unsigned long long)h->n_lanes);
   mix((unsigned long long)h->has_stop);
+  // (seg: timed with the step in link segments; entries from before it are not looked at)
   char buf[sizeof(prop.name) + 48];
-  snprintf(buf, sizeof buf, "%s|sm%d|%016llx", prop.name, h->sm_count, hsh);
+  snprintf(buf, sizeof buf, "%s|sm%d|%016llx|seg", prop.name, h->sm_count, hsh);
   return buf;
 }
 
