@@ -1599,24 +1599,22 @@ int sim_step_timed(sim_handle* h, int32_t n_steps, float* kernel_ms) {
   if (!h->routed) return fail(h, SIM_ESTATE, "sim_step_timed before sim_route / sim_set_routes");
   if (int rc = check_horizon(h, n_steps)) return rc;
   for (int k = 0; k < kNumKernels; k++) kernel_ms[k] = 0.0f;
-  if (n_steps > 0 && h->n_lanes >= kSegLanes && seg_possible(h) && seg_sized(h)) {
+  const long long t_end = h->t_host + n_steps;
+  while (n_steps > 0 && h->n_lanes >= kSegLanes && seg_possible(h) && seg_sized(h)) {
     if (int rc = seg_from_sorted(h)) return rc;
-  } else if (int rc = seg_to_sorted(h)) {
-    return rc;
-  }
-  if (h->seg) {
-    const long long t_end = h->t_host + n_steps;
+    if (!h->seg) break;
     float ms[2] = {0.0f, 0.0f};
     CK(launch_seg_steps_timed(h->d, h->grid, h->stream, n_steps, ms));
     h->pack_age = 1 << 20;
-    kernel_ms[kKFront] = ms[0];
-    kernel_ms[kKChunk] = ms[1];
+    kernel_ms[kKFront] += ms[0];
+    kernel_ms[kKChunk] += ms[1];
     if (int rc = check_device(h)) return rc;
     if (h->t_host == t_end) return SIM_OK;
-    // a segment was full: the rest in the sorted form
-    if (int rc = seg_regrow(h, 2)) return rc;
+    // a segment was full: the rest in larger ones or in the sorted form
+    if (int rc = seg_regrow(h, h->mirror->c.grow)) return rc;
     n_steps = (int)(t_end - h->t_host);
   }
+  if (int rc = seg_to_sorted(h)) return rc;
   float rest[kNumKernels];
   CK(launch_steps_timed(h->d, h->grid, h->has_stop, h->stream, n_steps, rest));
   for (int k = 0; k < kNumKernels; k++) kernel_ms[k] += rest[k];
@@ -2057,11 +2055,11 @@ int sim_adjoint(sim_handle* h, const sim_loss_spec* spec, double* grad_out, doub
     e = cudaMemcpyAsync(&h->mirror->c, h->d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e == cudaSuccess && h->mirror->c.grow) {
-      // a segment was full on the way: again from the start in the sorted form
+      // a segment was full on the way: again from the start in the sorted form (for this call:
+      // the next steps make larger segments)
       e = ckpt_copy(h, ck, false);
       if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->grow, 0, sizeof(int), h->stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(&h->d.ctl->loss, 0, 8, h->stream);
-      h->seg_off = true;
       forward();
     }
   }
@@ -2188,6 +2186,11 @@ int sim_autotune(sim_handle* h, int32_t trial_steps, const char* cache_path, sim
   int rc = dalloc(h, &ck, CL.bytes);
   if (rc) return rc;
   const sim_exec orig = h->exec;
+  const bool seg_off = h->seg_off;   // what fills up in a trial does not count after it
+  auto restore = [&]() {
+    h->seg_off = seg_off;
+    return ckpt_copy(h, ck, false);
+  };
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -2196,10 +2199,10 @@ int sim_autotune(sim_handle* h, int32_t trial_steps, const char* cache_path, sim
   for (const sim_exec& c : cand) {
     if (err != cudaSuccess) break;
     if (sim_set_exec(h, &c) != SIM_OK) continue;
-    err = ckpt_copy(h, ck, false);
+    err = restore();
     if (err != cudaSuccess) break;
     if ((rc = sim_step(h, trial_steps))) break;   // warm-up (builds the graphs of this step count)
-    err = ckpt_copy(h, ck, false);
+    err = restore();
     if (err != cudaSuccess) break;
     // the steps alone are timed: the restored state is in the sorted form, and graphs of eight
     // steps are otherwise captured in the course of a run
@@ -2216,7 +2219,7 @@ int sim_autotune(sim_handle* h, int32_t trial_steps, const char* cache_path, sim
       best = c;
     }
   }
-  if (err == cudaSuccess && !rc) err = ckpt_copy(h, ck, false);
+  if (err == cudaSuccess && !rc) err = restore();
   if (err == cudaSuccess) err = cudaStreamSynchronize(h->stream);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -111,3 +111,29 @@ def test_sample_of_a_step_that_did_not_fit(G, most, depart, how):
     g.step_timed(12) if how == "timed" else g.step(12)
     compare(g, o, "filled")
     compare_outputs(g, o, 7, "filled")
+
+
+# a segment that ran full in a call that times, taps or tries steps does not keep later steps out
+# of the segments (2 launches a step there, 7 in the sorted form)
+@pytest.mark.parametrize("call", ["timed", "adjoint", "autotune"])
+def test_full_segment_is_forgotten(G, call):
+    import oracle
+    sc, L = filling_link(1022 if call == "autotune" else 84, 7 if call == "autotune" else 1)
+    g, o = setup_pair(sc, G.Sim, oracle.OracleSim)
+    if call == "timed":
+        g.step_timed(4)
+        o.step(4)
+    elif call == "adjoint":
+        tgt = np.full((2, sc["demand"]["n_trips"]), 100.0)
+        grad, loss = g.adjoint(10, 5, tgt, 1)
+        og, oloss = o.adjoint(10, 5, tgt, 1)
+        assert abs(loss - oloss) <= 1e-12 * oloss
+        assert np.allclose(grad, np.reshape(og, (1, 5)), rtol=1e-9, atol=1e-9 * np.abs(og).max())
+    else:
+        g.autotune(10)   # back to the state before the link runs full
+        g.set_exec(mode=0)
+    n0 = g.launch_count()
+    g.step(4)
+    assert g.launch_count() - n0 == 2 * 4
+    o.step(4)
+    compare(g, o, call)
