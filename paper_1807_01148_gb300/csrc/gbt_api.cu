@@ -1052,108 +1052,126 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
   // link costs at most 1e6.
   const int delta = (int)std::max<long long>(1, 8 * csum / std::max(1, nl));
 
-  // eight trees in flight per SM (one per 256-thread block): a tree's rounds are short and
-  // synchronous, so more trees hide more of their latency (12,000 metro trees 49 ms with
-  // four, 43 with eight); four where the memory cap does not leave room for more
-  int n_cta = std::max(1, std::min<int>((int)origins.size(), h->sm_count * 8));
-  std::vector<void*> tmp;
-  auto talloc = [&](auto** p, size_t n) -> int {
-    int rc = dalloc(h, p, n);
-    if (!rc) tmp.push_back(*p);
-    return rc;
-  };
-  auto cleanup = [&]() {
-    for (void* p : tmp) dfree(h, p);
-    tmp.clear();
-  };
-
   RouteDev R{};
   int rc = SIM_OK;
-  int32_t *dos, *dis, *dil, *dorig, *dts, *dtl, *ddest;
-  int2 *doe, *die;
-  if ((rc = talloc(&dos, os.size())) || (rc = talloc(&doe, oe.size())) || (rc = talloc(&dis, is.size())) ||
-      (rc = talloc(&die, ie.size())) || (rc = talloc(&dil, il.size())) ||
-      (rc = talloc(&dorig, origins.size() + 1)) || (rc = talloc(&dts, ts.size())) ||
-      (rc = talloc(&dtl, tl.size())) || (rc = talloc(&ddest, (size_t)std::max(1, nt)))) {
+  // the call's device memory: tables, links by node, search arrays
+  std::vector<void*> tables, links, search;
+  auto get = [&](std::vector<void*>& part, auto** p, size_t n, const void* src = nullptr) {
+    if (rc) return;
+    std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(*p)>>>* q = nullptr;
+    if ((rc = dalloc(h, &q, n))) return;
+    part.push_back(q);
+    *p = q;
+    if (src && n) cudaMemcpy(q, src, n * sizeof(*q), cudaMemcpyHostToDevice);
+  };
+  auto drop = [&](std::vector<void*>& part) {
+    for (void* p : part) dfree(h, p);
+    part.clear();
+  };
+  auto cleanup = [&]() {
+    drop(tables);
+    drop(links);
+    drop(search);
+  };
+  // The links of a node as (node, cost) pairs, 20 bytes per link with the ids, or by id through
+  // arrays per link, 16.
+  bool pairs = true;
+  auto get_links = [&]() {
+    rc = SIM_OK;
+    if (pairs) {
+      get(links, &R.out_edge, oe.size(), oe.data());
+      get(links, &R.in_edge, ie.size(), ie.data());
+    } else {
+      std::vector<int32_t> ol((size_t)nl), fo(os.begin(), os.end() - 1);
+      for (int e = 0; e < nl; e++) ol[fo[h->lfrom[e]]++] = e;
+      get(links, &R.out_link, ol.size(), ol.data());
+      get(links, &R.lto, (size_t)nl, h->lto.data());
+      get(links, &R.cost, (size_t)nl, cost.data());
+      R.out_edge = R.in_edge = nullptr;
+    }
+    if (rc) drop(links);
+    return rc;
+  };
+  // Eight trees in flight per SM (one per 256-thread block): a tree's rounds are short and
+  // synchronous, so more trees hide more of their latency (12,000 metro trees 49 ms with
+  // four, 43 with eight).
+  int trees = 8, n_cta = 0;
+  auto get_search = [&]() {
+    rc = SIM_OK;
+    n_cta = std::max(1, std::min<int>((int)origins.size(), h->sm_count * trees));
+    const size_t per = (size_t)n_cta * (size_t)nn;
+    get(search, &R.node, per);
+    for (int32_t** q : {&R.qa, &R.qb, &R.fa, &R.fb}) get(search, q, per);
+    get(search, &R.cta_round, (size_t)n_cta);
+    get(search, &R.cta_epoch, (size_t)n_cta);
+    if (rc) {
+      drop(search);
+      return rc;
+    }
+    // distances beyond every epoch; the queue tags of -1 equal no round and no epoch (both
+    // count up from 1)
+    cudaMemset(R.node, 0xFF, per * sizeof(RouteNode));
+    cudaMemset(R.cta_round, 0, (size_t)n_cta * 4);
+    cudaMemset(R.cta_epoch, 0, (size_t)n_cta * 4);
+    return rc;
+  };
+  // Less of it where the rest does not fit beside it: four trees, then links by id.
+  auto shrink = [&]() {
+    cudaGetLastError();
+    if (trees > 4) {
+      trees = 4;
+      if (search.empty()) return true;
+      drop(search);
+      return get_search() == SIM_OK;
+    }
+    if (pairs) {
+      pairs = false;
+      if (links.empty()) return true;
+      drop(links);
+      return get_links() == SIM_OK;
+    }
+    return false;
+  };
+  auto with_room = [&](auto alloc) {
+    while ((rc = alloc()) == SIM_ENOMEM && shrink()) {}
+    return rc;
+  };
+  get(tables, &R.out_start, os.size(), os.data());
+  get(tables, &R.in_start, is.size(), is.data());
+  get(tables, &R.in_link, il.size(), il.data());
+  get(tables, &R.origins, origins.size() + 1);
+  if (!rc && !origins.empty())
+    cudaMemcpy(const_cast<int32_t*>(R.origins), origins.data(), origins.size() * 4, cudaMemcpyHostToDevice);
+  get(tables, &R.otrip_start, ts.size(), ts.data());
+  get(tables, &R.otrip_list, tl.size(), tl.data());
+  get(tables, &R.dest, (size_t)std::max(1, nt));
+  if (!rc && nt) cudaMemcpy(const_cast<int32_t*>(R.dest), h->dest.data(), (size_t)nt * 4, cudaMemcpyHostToDevice);
+  get(tables, &R.work, 1);
+  if (rc || with_room(get_links) || with_room(get_search)) {
     cleanup();
     return rc;
   }
-  cudaMemcpy(dos, os.data(), os.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(doe, oe.data(), oe.size() * 8, cudaMemcpyHostToDevice);
-  cudaMemcpy(dis, is.data(), is.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(die, ie.data(), ie.size() * 8, cudaMemcpyHostToDevice);
-  cudaMemcpy(dil, il.data(), il.size() * 4, cudaMemcpyHostToDevice);
-  if (!origins.empty()) cudaMemcpy(dorig, origins.data(), origins.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dts, ts.data(), ts.size() * 4, cudaMemcpyHostToDevice);
-  cudaMemcpy(dtl, tl.data(), tl.size() * 4, cudaMemcpyHostToDevice);
-  if (nt) cudaMemcpy(ddest, h->dest.data(), (size_t)nt * 4, cudaMemcpyHostToDevice);
-  RouteNode* dnode;
-  int32_t *qa, *qb, *fa, *fb, *cround;
-  unsigned* cep;
-  int* work;
-  const size_t n_tables = tmp.size();
-  for (;;) {
-    const size_t per = (size_t)n_cta * (size_t)nn;
-    rc = SIM_OK;
-    if ((rc = talloc(&dnode, per)) || (rc = talloc(&qa, per)) || (rc = talloc(&qb, per)) || (rc = talloc(&fa, per)) ||
-        (rc = talloc(&fb, per)) || (rc = talloc(&cround, (size_t)n_cta)) || (rc = talloc(&cep, (size_t)n_cta)) ||
-        (rc = talloc(&work, 1))) {
-      if (rc == SIM_ENOMEM && n_cta > h->sm_count * 4) {
-        cudaGetLastError();
-        n_cta = h->sm_count * 4;
-        while (tmp.size() > n_tables) {
-          dfree(h, tmp.back());
-          tmp.pop_back();
-        }
-        continue;
-      }
-      cleanup();
-      return rc;
-    }
-    break;
-  }
-  const size_t per = (size_t)n_cta * (size_t)nn;
-  // distances beyond every epoch; the queue tags of -1 equal no round and no epoch (both
-  // count up from 1)
-  cudaMemset(dnode, 0xFF, per * sizeof(RouteNode));
-  cudaMemset(cround, 0, (size_t)n_cta * 4);
-  cudaMemset(cep, 0, (size_t)n_cta * 4);
   R.nn = nn;
   R.nl = nl;
-  R.out_start = dos;
-  R.out_edge = doe;
-  R.in_start = dis;
-  R.in_edge = die;
-  R.in_link = dil;
-  R.origins = dorig;
+  R.lfrom = h->d.lfrom;
   R.n_origins = (int)origins.size();
-  R.otrip_start = dts;
-  R.otrip_list = dtl;
-  R.dest = ddest;
-  R.node = dnode;
-  R.qa = qa;
-  R.qb = qb;
-  R.fa = fa;
-  R.fb = fb;
-  R.cta_epoch = cep;
-  R.cta_round = cround;
   R.roff = const_cast<int32_t*>(h->d.roff);
   R.rlen = const_cast<int32_t*>(h->d.rlen);
-  R.work = work;
   R.delta = delta;
   R.ctl = h->d.ctl;
   if (flow) {
     // counts on a scratch control block, so that the simulation's counters stay intact
     Ctl* fctl;
-    if ((rc = talloc(&fctl, 1))) {
+    if (with_room([&]() { return dalloc(h, &fctl, 1); })) {
       cleanup();
       return rc;
     }
+    tables.push_back(fctl);
     R.ctl = fctl;
     R.routes = nullptr;
     R.cap = 0;
     R.flow = flow;
-    cudaMemset(work, 0, 4);
+    cudaMemset(R.work, 0, 4);
     cudaMemset(fctl, 0, sizeof(Ctl));
     cudaMemset(flow, 0, (size_t)std::max(1, nl) * 4);
     if (cudaDeviceSynchronize() != cudaSuccess) {
@@ -1189,7 +1207,7 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
   for (int attempt = 0; attempt < 2; attempt++) {
     dfree(h, h->routes);
     h->routes = nullptr;
-    if ((rc = dalloc(h, &h->routes, cap))) {
+    if (with_room([&]() { return dalloc(h, &h->routes, cap); })) {
       dfree(h, old_routes);
       if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
@@ -1198,7 +1216,7 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     if (kept) cudaMemcpy(h->routes, old_routes, kept * 4, cudaMemcpyDeviceToDevice);
     R.routes = h->routes;
     R.cap = cap;
-    cudaMemset(work, 0, 4);
+    cudaMemset(R.work, 0, 4);
     cudaMemset(h->d.ctl, 0, sizeof(Ctl));
     if (kept) cudaMemcpy(&h->d.ctl->route_cursor, &kept, sizeof(kept), cudaMemcpyHostToDevice);
     if (cudaDeviceSynchronize() != cudaSuccess) {

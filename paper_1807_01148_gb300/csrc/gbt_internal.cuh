@@ -323,9 +323,10 @@ struct __align__(16) RouteNode {
 struct RouteDev {
   int nn, nl;
   const int32_t* out_start;
-  const int2* out_edge;         // by tail node: (head, cost); null: the three arrays below
+  const int2* out_edge;         // by tail node: (head, cost); null: no pairs, the arrays per link instead
   const int32_t* out_link;      // by tail node: link ids
-  const int32_t* lto;           // per link
+  const int32_t* lfrom;         // per link
+  const int32_t* lto;
   const int32_t* cost;
   const int32_t* in_start;
   const int2* in_edge;          // by head node, ascending link id: (tail, cost)

@@ -44,7 +44,7 @@ __device__ __forceinline__ int dval(const RouteNode* node, int v, unsigned hi) {
 // Walk from v (distance dv) back to o by the eight threads of a group.  Returns the number
 // of links, -1 when no tight in-link is found; sink(j, link) is called by one of the threads
 // for the j-th link from the end.
-template <typename Sink>
+template <bool PACKED, typename Sink>
 __device__ __forceinline__ int walk_back(const RouteDev& R, const RouteNode* node, unsigned hi, int o, int v, int dv,
                                          Sink sink) {
   const int lane = threadIdx.x & 31, gl = lane & (kWalkLanes - 1), g0 = lane - gl;
@@ -57,7 +57,13 @@ __device__ __forceinline__ int walk_back(const RouteDev& R, const RouteNode* nod
       p = p0 + gl;
       bool ok = false;
       if (p < e) {
-        const int2 x = R.in_edge[p];
+        int2 x;
+        if (PACKED) {
+          x = R.in_edge[p];
+        } else {
+          const int l = R.in_link[p];
+          x = make_int2(R.lfrom[l], R.cost[l]);
+        }
         u = x.x;
         du = dval(node, u, hi);
         us = R.in_start[u];
@@ -78,8 +84,8 @@ __device__ __forceinline__ int walk_back(const RouteDev& R, const RouteNode* nod
   return n;
 }
 
-// PACKED: the out-links as (head, cost) pairs; otherwise as the caller's link arrays
-// (sim_sssp_static, which has no memory to pack them in).
+// PACKED: the links of a node as (node, cost) pairs; otherwise by id, through arrays per link
+// (sim_sssp_static, which has no memory to pack them in, and planning under a memory cap).
 template <bool PACKED>
 __global__ void __launch_bounds__(kRouteThreads) k_sssp_route(RouteDev R) {
   __shared__ int sh_oi, sh_nf, sh_nf2, sh_min;
@@ -227,7 +233,7 @@ __global__ void __launch_bounds__(kRouteThreads) k_sssp_route(RouteDev R) {
       const int dd = dval(node, d, hi);
       int n = -1;
       if (dd != INT_MAX)
-        n = walk_back(R, node, hi, o, d, dd, [&](int j, int link) {
+        n = walk_back<PACKED>(R, node, hi, o, d, dd, [&](int j, int link) {
           if (R.flow) atomicAdd(&R.flow[link], 1u);
           else if (j < room) note[j] = link;
         });
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(kRouteThreads) k_sssp_route(RouteDev R) {
         for (int j = gl; j < n; j += kWalkLanes) R.routes[off + (unsigned)(n - 1 - j)] = note[j];
         __syncwarp(gm);   // read before the next trip's walk writes
       } else {
-        walk_back(R, node, hi, o, d, dd, [&](int j, int link) { R.routes[off + (unsigned)(n - 1 - j)] = link; });
+        walk_back<PACKED>(R, node, hi, o, d, dd, [&](int j, int link) { R.routes[off + (unsigned)(n - 1 - j)] = link; });
       }
     }
   }

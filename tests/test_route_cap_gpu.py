@@ -1,0 +1,50 @@
+"""Trip planning under a device-memory cap (sim_params.max_device_bytes)."""
+import numpy as np
+import pytest
+
+from paper_1807_01148_gb300 import scenarios as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_1807_01148_gb300 import gbtraffic
+    return gbtraffic
+
+
+def _capped(sc, cap):
+    return dict(sc, params=dict(sc["params"], max_device_bytes=cap))
+
+
+def _least(G, sc, lo=1 << 10, hi=1 << 28):
+    """The least cap under which the handle can be created."""
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        try:
+            G.Sim(_capped(sc, mid)).close()
+            hi = mid
+        except G.SimError:
+            lo = mid
+    return hi
+
+
+def _planning(sc, trees):
+    """Bytes that planning needs at least: link arrays of 4 words per link, the nodes' tables, 32
+    bytes per node and tree in flight, 96 links per trip."""
+    nn, nl, nt = sc["network"]["n_nodes"], len(sc["network"]["link_from"]), sc["demand"]["n_trips"]
+    n_org = len(np.unique(sc["demand"]["origin"]))
+    n_cta = min(n_org, trees)
+    return (4 * (4 * nl + 3 * (nn + 1) + n_org + 1 + 2 * nt) + n_cta * (32 * nn + 8) + 4
+            + 4 * max(1024, 96 * nt))
+
+
+@pytest.mark.parametrize("room", [0, 4, 1 << 20], ids=["links by id", "by id, a little more", "pairs"])
+def test_least_room(G, room):
+    import oracle
+    sc = S.small_grid(n=20, n_trips=200, steps=100)
+    g, o = G.Sim(_capped(sc, _least(G, sc) + _planning(sc, 1 << 30) + room)), oracle.OracleSim(sc)
+    g.route()
+    o.route()
+    (go, gl), (oo, ol) = g.routes(), o.routes()
+    assert np.array_equal(go, oo) and np.array_equal(gl, ol)
