@@ -185,6 +185,7 @@ struct sim_handle {
   bool graph_seg = false, pgraph_seg = false, tape_graph_seg = false;   // form of the captured graphs
   std::vector<void*> seg_mem;
   bool seg_building = false;   // seg_alloc is under way
+  bool seg_keep = false;       // an allocation that can do with less is tried: the segments stay
 };
 
 namespace {
@@ -291,7 +292,7 @@ int seg_to_sorted(sim_handle* h) {
 // Give the segments' memory back (the state goes on in the sorted form until it is next
 // replaced).  False when there is none to give.
 bool seg_release(sim_handle* h) {
-  if (h->seg_building || h->seg_mem.empty()) return false;
+  if (h->seg_building || h->seg_keep || h->seg_mem.empty()) return false;
   h->seg_off = true;
   if (seg_to_sorted(h) != SIM_OK || cudaStreamSynchronize(h->stream) != cudaSuccess) return false;
   seg_free(h);
@@ -1115,7 +1116,10 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     cudaMemset(R.cta_epoch, 0, (size_t)n_cta * 4);
     return rc;
   };
-  // Less of it where the rest does not fit beside it: four trees, then links by id.
+  // Less of it where the rest does not fit beside it: four trees; then without the segments of
+  // the running state (an assignment goes on with it, and it would step in the sorted form until
+  // it is next replaced); then links by id.
+  bool keep = true;
   auto shrink = [&]() {
     cudaGetLastError();
     if (trees > 4) {
@@ -1123,6 +1127,10 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
       if (search.empty()) return true;
       drop(search);
       return get_search() == SIM_OK;
+    }
+    if (keep) {
+      keep = false;
+      return true;
     }
     if (pairs) {
       pairs = false;
@@ -1133,7 +1141,11 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     return false;
   };
   auto with_room = [&](auto alloc) {
-    while ((rc = alloc()) == SIM_ENOMEM && shrink()) {}
+    do {
+      h->seg_keep = keep;
+      rc = alloc();
+      h->seg_keep = false;
+    } while (rc == SIM_ENOMEM && shrink());
     return rc;
   };
   get(tables, &R.out_start, os.size(), os.data());

@@ -48,3 +48,22 @@ def test_least_room(G, room):
     o.route()
     (go, gl), (oo, ol) = g.routes(), o.routes()
     assert np.array_equal(go, oo) and np.array_equal(gl, ol)
+
+
+def test_assignment_keeps_the_segments(G):
+    # beside the segments (about 20 MB) there is room for four trees per SM, not for eight: the
+    # running state stays in the segments (2 launches a step, 7 in the sorted form)
+    import torch
+    sc = S.small_grid(n=40, n_trips=8000, steps=100)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert len(np.unique(sc["demand"]["origin"])) > 8 * sms
+    g = G.Sim(_capped(sc, _least(G, sc) + _planning(sc, 4 * sms) + (30 << 20)))
+    g.route()
+    g.step(4)
+    n0 = g.launch_count()
+    g.step(4)
+    assert g.launch_count() - n0 == 2 * 4
+    g.assign_static(np.full(len(sc["network"]["link_from"]), 1800.0), max_iter=1)
+    n0 = g.launch_count()
+    g.step(4)
+    assert g.launch_count() - n0 == 2 * 4
