@@ -185,6 +185,7 @@ struct sim_handle {
   bool graph_seg = false, pgraph_seg = false, tape_graph_seg = false;   // form of the captured graphs
   std::vector<void*> seg_mem;
   bool seg_building = false;   // seg_alloc is under way
+  size_t seg_need = 0;         // bytes of the segments for the present vehicle types (0: not known)
   bool seg_keep = false;       // an allocation that can do with less is tried: the segments stay
 };
 
@@ -310,6 +311,9 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   float vmin = d.vlen;
   for (float v : h->vty_len) vmin = std::min(vmin, v);
   if (h->n_lanes >= 1 << 26) return fail(h, SIM_ENOMEM, "lane ids beyond 26 bits");   // slots are packed with flags
+  // known not to fit the cap: no tables are made for that (a state may be written often)
+  auto over = [&](size_t need) { return h->max_bytes && h->bytes + need > h->max_bytes; };
+  if (!now && over(h->seg_need)) return fail(h, SIM_ENOMEM, "device memory cap (sim_params.max_device_bytes) reached");
   std::vector<int32_t> cap;
   seg_capacities(nl, h->len.data(), h->lanes.data(), h->nt, vmin, now, cap);
   std::vector<int32_t> lslot;
@@ -344,9 +348,35 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   }
   for (int e = 0; e < nl; e++)
     for (int l = 0; l < h->lanes[e]; l++) tail[(size_t)lslot[e] + l] = start[h->lfrom[e]];
-  h->seg_building = true;
+  auto all = [&](auto&& get) {
+    get(&d.rec, (size_t)total);
+    get(&d.rng, ns);
+    get(&d.sinfo, ns, pad.data());
+    get(&d.slot_to, ns);
+    get(&d.lane_seg, ns, seg.data());
+    get(&d.lstat, ns, none.data());
+    get(&d.rear2, ns * 2);
+    get(&d.best2, ns);
+    get(&d.fres, ns);
+    get(&d.cr2, ns);
+    get(&d.lnext, (size_t)nl, lnext.data());
+    get(&d.lslot, (size_t)nl, lslot.data());
+    get(&d.stail, ns, tail.data());
+    get(&d.nin_slot, (size_t)nl, nin.data());
+    get(&d.qnext, ns);
+    get(&d.big_links, (size_t)std::max(1, n_big));
+    get(&d.tl, (size_t)nl * 32);   // a run has one link at least
+    get(&d.late, (size_t)nl);
+    get(&d.listed, (size_t)nl);
+    get(&d.cuts, ns / 32);
+  };
+  size_t need = 0;
+  all([&](auto** p, size_t n, const void* = nullptr) { need += std::max<size_t>(1, n) * sizeof(**p); });
+  if (!now) h->seg_need = need;
   int rc = SIM_OK;
-  auto get = [&](auto** p, size_t n, const void* src = nullptr) {
+  if (over(need)) return fail(h, SIM_ENOMEM, "device memory cap (sim_params.max_device_bytes) reached");
+  h->seg_building = true;
+  all([&](auto** p, size_t n, const void* src = nullptr) {
     if (rc) return;
     std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(*p)>>>* q = nullptr;
     if ((rc = dalloc(h, &q, n))) return;
@@ -354,27 +384,7 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
     *p = q;
     if (src && n && cudaMemcpyAsync(q, src, n * sizeof(*q), cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
       rc = fail(h, SIM_ECUDA, "segment tables");
-  };
-  get(&d.rec, (size_t)total);
-  get(&d.rng, ns);
-  get(&d.sinfo, ns, pad.data());
-  get(&d.slot_to, ns);
-  get(&d.lane_seg, ns, seg.data());
-  get(&d.lstat, ns, none.data());
-  get(&d.rear2, ns * 2);
-  get(&d.best2, ns);
-  get(&d.fres, ns);
-  get(&d.cr2, ns);
-  get(&d.lnext, (size_t)nl, lnext.data());
-  get(&d.lslot, (size_t)nl, lslot.data());
-  get(&d.stail, ns, tail.data());
-  get(&d.nin_slot, (size_t)nl, nin.data());
-  get(&d.qnext, ns);
-  get(&d.big_links, (size_t)std::max(1, n_big));
-  get(&d.tl, (size_t)nl * 32);   // a run has one link at least
-  get(&d.late, (size_t)nl);
-  get(&d.listed, (size_t)nl);
-  get(&d.cuts, ns / 32);
+  });
   if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(h, SIM_ECUDA, "segment tables");
   h->seg_building = false;
   if (rc) {
@@ -1865,6 +1875,7 @@ int sim_set_vehicle_types(sim_handle* h, int32_t n_types, const sim_vehicle_type
   h->vty_len.clear();
   h->vty_ascale.clear();
   h->vty_vmax.clear();
+  h->seg_need = 0;   // shorter vehicles, longer segments
   h->graph_dirty = true;
   h->pgraph_n = -1;
   h->tape_graph_dirty = true;

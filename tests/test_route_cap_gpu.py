@@ -1,8 +1,12 @@
-"""Trip planning under a device-memory cap (sim_params.max_device_bytes)."""
+"""Trip planning and written states under a device-memory cap (sim_params.max_device_bytes)."""
+import time
+
 import numpy as np
 import pytest
 
 from paper_1807_01148_gb300 import scenarios as S
+
+from .test_seg_gpu import _grid
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +71,25 @@ def test_assignment_keeps_the_segments(G):
     n0 = g.launch_count()
     g.step(4)
     assert g.launch_count() - n0 == 2 * 4
+
+
+def test_written_state_without_room_for_segments(G):
+    # finding no room for the segments costs a written state no more than laying them out does
+    sc = _grid(n=128, lanes=3, n_trips=2000)
+    n = sc["demand"]["n_trips"]
+    st = dict(status=np.zeros(n, np.uint8), link=np.zeros(n, np.int32), lane=np.zeros(n, np.int32),
+              cursor=np.zeros(n, np.int32), x=np.zeros(n, np.float32), v=np.zeros(n, np.float32))
+    took = []
+    for cap in (0, _least(G, sc) + (4 << 20)):
+        g = G.Sim(_capped(sc, cap))
+        g.set_routes(sc["routes"]["offsets"], sc["routes"]["links"])
+        one = []
+        for _ in range(12):
+            t = time.perf_counter()
+            g.write_state(st)
+            one.append(time.perf_counter() - t)
+        took.append(np.median(one))
+        n0 = g.launch_count()
+        g.step(4)
+        assert g.launch_count() - n0 == (2 * 4 + 1, 7 * 4)[cap > 0]
+    assert took[1] < 2.0 * took[0], took
