@@ -1215,6 +1215,7 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     return SIM_OK;
   }
   // the kept routes (subset mode) stay at the front of the store, new ones follow
+  h->routed = false;   // until the new ones are there: a failure below leaves none
   int32_t* old_routes = nullptr;
   unsigned long long kept = 0;
   if (sel) {
@@ -1231,7 +1232,6 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     h->routes = nullptr;
     if (with_room([&]() { return dalloc(h, &h->routes, cap); })) {
       dfree(h, old_routes);
-      if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
       return rc;
     }
@@ -1243,7 +1243,6 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     if (kept) cudaMemcpy(&h->d.ctl->route_cursor, &kept, sizeof(kept), cudaMemcpyHostToDevice);
     if (cudaDeviceSynchronize() != cudaSuccess) {
       dfree(h, old_routes);
-      if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
       return fail(h, SIM_ECUDA, "route setup failed");
     }
@@ -1251,7 +1250,6 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     cudaError_t e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
       dfree(h, old_routes);
-      if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
       return cuda_fail(h, e, "route kernel");
     }
@@ -1259,7 +1257,6 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     cudaMemcpy(&c, h->d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost);
     if (c.err & kErrUnreach) {
       dfree(h, old_routes);
-      if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
       char buf[96];
       snprintf(buf, sizeof buf, "trip %d: destination unreachable", c.err_info);
@@ -1267,7 +1264,6 @@ int route_impl(sim_handle* h, const int32_t* link_cost_ds, const std::vector<uin
     }
     if (c.err) {
       dfree(h, old_routes);
-      if (sel) h->routed = false;   // the kept routes are gone with the failed store
       cleanup();
       return fail(h, SIM_EDEVICE, "route extraction failed");
     }
@@ -1367,6 +1363,7 @@ int sim_set_routes(sim_handle* h, const int32_t* offsets, const int32_t* links) 
     len[i] = offsets[i + 1] - offsets[i];
     h->long_route = h->long_route || len[i] >= kMaxRem;
   }
+  h->routed = false;   // until the new ones are there
   dfree(h, h->routes);
   h->routes = nullptr;
   int rc = dalloc(h, &h->routes, (size_t)std::max<long long>(1, total));

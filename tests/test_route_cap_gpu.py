@@ -6,6 +6,7 @@ import pytest
 
 from paper_1807_01148_gb300 import scenarios as S
 
+from .parity import run_lockstep
 from .test_seg_gpu import _grid
 
 pytestmark = pytest.mark.gpu
@@ -93,3 +94,24 @@ def test_written_state_without_room_for_segments(G):
         g.step(4)
         assert g.launch_count() - n0 == (2 * 4 + 1, 7 * 4)[cap > 0]
     assert took[1] < 2.0 * took[0], took
+
+
+def test_routes_that_do_not_fit_leave_none(G):
+    # the old routes are gone by then: stepping is refused until there are new ones
+    import oracle
+    sc = _grid(n=24, n_trips=3000)
+    short = sc["routes"]
+    off, links = S.random_walk_routes(sc, 400, 600, seed=S.BASE_SEED)
+    g = G.Sim(_capped(sc, _least(G, sc) + (1 << 20)))
+    g.set_routes(short["offsets"], short["links"])
+    g.step(10)
+    with pytest.raises(G.SimError) as e:
+        g.set_routes(off, links)
+    assert e.value.code == G.SIM_ENOMEM
+    with pytest.raises(G.SimError) as e:
+        g.step(1)
+    assert e.value.code == G.SIM_ESTATE
+    g.set_routes(short["offsets"], short["links"])
+    o = oracle.OracleSim(sc)
+    o.set_routes(short["offsets"], short["links"])
+    run_lockstep(g, o, 20, 10, check_occ=False)
