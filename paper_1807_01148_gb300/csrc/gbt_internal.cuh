@@ -284,8 +284,8 @@ constexpr int kPackSteps = 8;   // steps that the packed lists hold for
 struct SegDev : Dev {
   VehRec* rec;                     // link e owns cap records from its segment's start on, in (lane, x, vid) order
   uint32_t* rng;                   // per slot: its vehicles, start relative to the segment | count << 16 (rng_start,
-                                   // rng_count) | 1 << 31 where a whole block wrote it in this step's move phase
-                                   // (rng_done; the next front phase takes the mark out)
+                                   // rng_count) | 2 + parity of the step << 30 where a whole block wrote it; the next
+                                   // step's move phase writes the lane anew or takes the mark out
   const uint32_t* sinfo;           // per slot: LaneStat::info (control 3: empty slot)
   const int2* lane_seg;            // per slot: its link's segment start and capacity
   const LaneStat* lstat;           // per slot

@@ -86,8 +86,6 @@ __device__ __forceinline__ bool seg_big(int vehicles, int lanes) { return vehicl
 // Fields of SegDev::rng.
 __device__ __forceinline__ int rng_start(uint32_t r) { return (int)(r & 0xffffu); }
 __device__ __forceinline__ int rng_count(uint32_t r) { return (int)(r >> 16 & 0x3fffu); }
-constexpr uint32_t kRngDone = 1u << 31;
-__device__ __forceinline__ bool rng_done(uint32_t r) { return (r & kRngDone) != 0; }
 
 __device__ __forceinline__ bool seg_stopped(const SegDev& d) {
   const int err = d.ctl->err, grow = d.ctl->grow;   // (cached: see step_timed_out)
@@ -256,6 +254,7 @@ __device__ __forceinline__ void seg_pack(const SegDev& d, SegPack* packs, int ba
     }
     n += __popc(m);
     veh += __shfl_sync(0xffffffffu, inc, 31);
+    if (r >> 30) d.rng[g] = r & 0x3fffffffu;   // a block's mark: the lists may leave the link out (see seg_move)
   }
   __syncwarp();
   // as many links as stay within the limits, at least one (a link has at most 8 lanes, so
@@ -333,7 +332,6 @@ __device__ __forceinline__ void seg_front(const SegDev& d, int t) {
     const int g = d.packed ? d.tl[k] : k;
     if (g < 0) continue;
     const uint32_t r = d.rng[g];
-    if (rng_done(r)) d.rng[g] = r & ~kRngDone;   // an earlier step's
     const int cnt = rng_count(r), end = rng_start(r) + cnt;
     // (the slot's other arrays are loaded along with its range)
     const float4* ls = reinterpret_cast<const float4*>(d.lstat + g);
@@ -965,7 +963,7 @@ __device__ __forceinline__ void seg_run(const SegDev& d, SM& S, const SegLane& l
       const int s = inc - cnt - first;
       S.wb[tid] = S.sg[tid] + s;
       S.cn[tid] = cnt;
-      d.rng[S.gs[tid]] = (uint32_t)s | (uint32_t)cnt << 16 | (NT == 32 ? 0u : kRngDone);
+      d.rng[S.gs[tid]] = (uint32_t)s | (uint32_t)cnt << 16 | (NT == 32 ? 0u : 2u + (unsigned)(t & 1)) << 30;
     }
   }
   // a stayer not below the next stayer of its lane: the whole lane is ranked by counting
@@ -1070,7 +1068,7 @@ __device__ __forceinline__ SegLane seg_lane(const SegDev& d, int g, int t) {
   ln.fr = d.fres[g];
   ln.start = rng_start(r);
   ln.cnt = rng_count(r);
-  ln.done = rng_done(r);
+  ln.done = (r >> 30) == 2u + (unsigned)(t & 1);
   const unsigned info = __float_as_uint(ln.lb.z);
   if (ln.cnt == 0) ln.fr.y = 0;   // an empty lane's record is an older step's
   if (epoch_current(bk, t)) {
@@ -1205,6 +1203,8 @@ __device__ __forceinline__ void seg_move(const SegDev& d, unsigned char* smem, i
       }
       if (__any_sync(0xffffffffu, ln.on && (ln.cnt || ln.ext || ln.due)))
         seg_run<32, SegSmem, OUT, TYPES, TAPE>(d, S, ln, 32, t, s_cn);
+      else if (ln.on && d.rng[g])   // nothing here but the mark of a block that emptied the link in the
+        d.rng[g] = 0;               // step before; in the next step it would pass for that step's
       ja = jb;
     } while (ja < jend);
   }
