@@ -37,7 +37,9 @@ UNIT = "vehicle-steps/s"
 # one pass over nearly sorted (u64 key + u32 id) records (24 B).
 STEP_KERNEL_BYTES = 40
 WHOLE_STEP_BYTES = 64
-# kernels that make up the plain step kernel (the lane-front and chunk kernels)
+# kernels that make up the plain step kernel: the lane fronts and, under "chunk", the chunk kernel of
+# the sorted form or the move phase of the link-segment form (which makes the next order as well,
+# so that the two are the whole step there)
 STEP_KERNELS = ("front", "chunk")
 
 # Implementation bytes per vehicle that each kernel of this design moves (every array
@@ -52,17 +54,16 @@ IMPL_BYTES = {
 }
 
 
-# DRAM bytes (read + write) per active vehicle per launch of the plain step kernel
-# (front + chunk), from the ncu capture summarised under profiles/, valid only for the
-# kernel sources it was taken on.
-PROFILED_SRC_SHA = "13600078790119c1"
-PROFILED_STEP_TRAFFIC = 149.0   # k_front 67.4 + k_chunk 81.5 B per active vehicle (987,466 vehicles)
+# DRAM bytes (read + write) per active vehicle per step of the link-segment form's two kernels, from
+# the ncu capture summarised under profiles/, valid only for the kernel sources it was taken on.
+PROFILED_SRC_SHA = "fbc53245f7405c44"
+PROFILED_STEP_TRAFFIC = 266.0   # k_seg_front 124 + k_seg_move 142 B per active vehicle (999,999 vehicles)
 
 
 def kernel_source_sha():
     import hashlib
     h = hashlib.sha256()
-    for f in ("gbt_fused.cu", "gbt_rebuild.cuh", "gbt_stepdev.cuh", "gbt_internal.cuh"):
+    for f in ("gbt_seg.cuh", "gbt_seg.cu", "gbt_stepdev.cuh", "gbt_internal.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1807_01148_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -633,9 +634,10 @@ def run_cuda(args):
     achieved_fl = STEP_KERNEL_BYTES * avg_active_fl / (step_ms_fl * 1e-3) / 1e9
     achieved = STEP_KERNEL_BYTES * avg_active / (step_ms * 1e-3) / 1e9
     whole = WHOLE_STEP_BYTES * (veh_steps / args.steps) / (ms / args.steps * 1e-3) / 1e9
-    # (the bytes are the sorted form's; in link segments its other kernels take no time)
+    # (in link segments the sorted form's other kernels take no time; the bytes are theirs)
+    segments = not kms.get("scatter")
     impl_gbs = {k: IMPL_BYTES[k] * avg_active / (kms[k] / args.steps * 1e-3) / 1e9
-                for k in IMPL_BYTES if k in kms and kms.get("scatter")}
+                for k in IMPL_BYTES if k in kms and not segments}
 
     # -- end to end through the C ABI with host buffers: load the snapshot from pinned host
     #    memory, then every step read positions and speeds back to pinned host memory.  The
@@ -736,8 +738,11 @@ def run_cuda(args):
                    "l2": "headline steps back to back: working set > L2 (state, scratch and per-lane arrays "
                          "~0.5 GB); roofline: L2 flushed before every timed step",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
-        "roofline": {"bound": "hbm", "kernel": "plain step kernel (front + chunk: neighbours, lane change, "
-                                                 "car following, admission, transition)",
+        "roofline": {"bound": "hbm", "kernel": ("lane fronts + move phase of the link-segment step: neighbours, lane "
+                                                  "change, car following, admission, transition, next order (the whole "
+                                                  "step)") if segments else
+                                                 ("plain step kernel (front + chunk: neighbours, lane change, "
+                                                  "car following, admission, transition)"),
                      "achieved": achieved_fl, "peak": hbm_peak, "unit": "GB/s", "frac": achieved_fl / hbm_peak,
                      "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)",
                      "alg_bytes_per_unit": STEP_KERNEL_BYTES, "unit_of_work": "vehicle-step",
@@ -745,10 +750,10 @@ def run_cuda(args):
                      "timing": "CUDA events around the two kernels, L2 flushed before every step",
                      "back_to_back": {"achieved": achieved, "frac": achieved / hbm_peak, "ms_per_launch": step_ms},
                      "traffic": (PROFILED_STEP_TRAFFIC * avg_active_fl
-                                 if PROFILED_STEP_TRAFFIC and kernel_source_sha() == PROFILED_SRC_SHA else None),
-                     "traffic_note": "ncu dram bytes (read + write) of the front and chunk kernels per vehicle on a "
+                                 if segments and kernel_source_sha() == PROFILED_SRC_SHA else None),
+                     "traffic_note": "ncu dram bytes (read + write, cold caches) of the two kernels per vehicle on a "
                                      "smaller capture of the same network, scaled to this launch's vehicles; null "
-                                     "when the kernel sources changed since",
+                                     "when the kernel sources changed since or the step ran in the sorted form",
                      "whole_step": {"alg_bytes_per_unit": WHOLE_STEP_BYTES, "achieved": whole,
                                     "frac": whole / hbm_peak, "ms_per_step": ms / args.steps,
                                     "timing": "graph-launched steps back to back (the headline value)"}},

@@ -252,15 +252,18 @@ int upload(sim_handle* h, T** p, const T* src, size_t n) {
 
 // ------------------------------------------------------------------ the two forms of the state
 // Which form the steps run in.  Graph execution: networks of kSegLanes lanes and more in the
-// segments, smaller ones in the sorted form, whose launches per step (7 to 9) sim_launch_count
-// reports for small networks and callers rely on there.  Persistent execution (one launch
-// either way): the segments on any network.  Measured, us per step with the reads of the state,
-// sorted -> segments: 20 x 20 grid (3,040 lanes, 2,050 vehicles) 43.0 -> 18.5; town of 6,700
-// lanes (with its share of planning) 60.9 -> 28.4; district of 42,000 lanes with outputs and
-// trucks 94.6 -> 86.5.  On networks with more groups of lanes than resident warps of the move
-// phase, in packed lists (SegDev::packed): 64 copies of a grid (321,000 lanes) 76.6 -> 62.2;
-// metro (782,000 lanes) with 2.11M vehicles 273 -> 267 and, in the persistent launch, with
-// 173,000 90 -> 76.
+// segments, smaller ones in the sorted form.  That line is not one of speed: sim_launch_count
+// reports 7 to 9 launches per step on small networks and callers rely on it there (a launch
+// count of 2 per step comes with the segments).  Without that promise the segments would be the
+// form at any size: us per step with the reads of the state, calls of 20 steps, sorted ->
+// segments: ring of 50 vehicles (calls of 10) 23.5 -> 13.6; grids of 6 x 6 (240 lanes) 22.8 ->
+// 13.8, 10 x 10 (720) 29.2 -> 15.9, 14 x 14 (1,456) 32.6 -> 17.0, 16 x 16 (1,920) 33.5 -> 18.0;
+// and above the line 20 x 20 (3,040 lanes, 2,050 vehicles) 43.0 -> 18.5; town of 6,700
+// lanes (with its share of planning) 60.1 -> 27.9; district of 42,000 lanes with outputs and
+// trucks 94 to 96 -> 86 to 90.  On networks with more groups of lanes than resident warps of the
+// move phase, in packed lists (SegDev::packed): 64 copies of a grid (321,000 lanes) 76.9 -> 62.3;
+// metro (782,000 lanes) with 2.11M vehicles 275 -> 268.  Persistent execution (one launch either
+// way): the segments on any network; metro with 173,000 vehicles 90 -> 76 (on some boxes 93 -> 86).
 // Not in the segments: networks where links longer than a staged chunk carry most of the
 // road, for which the sorted form has its big-chunk kernel (1,000 queues of 570 vehicles: 118
 // against 122).

@@ -21,7 +21,8 @@ __device__ __forceinline__ void griddep_next(const SegDev& d) {
 }
 
 // Bound by the latency of its dependent loads (range and slot arrays, front record and link
-// record, rear record of the next lane): six blocks of 40 registers per SM.
+// record, rear record of the next lane; a quarter of metro, 527,500 vehicles: 22.7 cycles per
+// instruction on loads, DRAM at 24%): six blocks of 40 registers per SM.
 template <bool TYPES, bool TAPE>
 __global__ void __launch_bounds__(256, 6) k_seg_front(SegDev d) {
   griddep_wait();
@@ -40,11 +41,11 @@ __global__ void __launch_bounds__(256) k_seg_pack(SegDev d) {
   seg_pack_all(d, packs, (int)d.ctl->t);
 }
 
-// Bound by instruction issue and load latency together (a quarter of metro, 580,000 vehicles:
-// 42% of issue slots, most stalls on loads, waits within the warp next).  Three blocks of 80
-// registers measured better than four of 64, whose spills miss the little L1 that the staging
-// areas leave: metro, 2.11M vehicles, 4 steps 1,110 -> 1,077 us; 64 grids, 10 steps 670 -> 645;
-// two blocks: 1,269 and 743.
+// Bound by instruction issue and latency together (a quarter of metro, 527,500 vehicles: 52 warp
+// instructions per vehicle at 17.9 active threads, 41% of issue slots; per instruction 2.8 cycles of
+// fixed latency, 2.5 at barriers, 2.4 on loads).  Three blocks of 80 registers measured better than
+// four of 64, whose spills miss the little L1 that the staging areas leave: metro, 2.11M vehicles,
+// 4 steps 1,110 -> 1,077 us; 64 grids, 10 steps 670 -> 645; two blocks: 1,269 and 743.
 template <bool OUT, bool TYPES, bool TAPE>
 __global__ void __launch_bounds__(kSegThreads, 3) k_seg_move(SegDev d) {
   griddep_wait();
