@@ -314,8 +314,10 @@ int seg_alloc(sim_handle* h, const int32_t* now) {
   float vmin = d.vlen;
   for (float v : h->vty_len) vmin = std::min(vmin, v);
   if (h->n_lanes >= 1 << 26) return fail(h, SIM_ENOMEM, "lane ids beyond 26 bits");   // slots are packed with flags
-  // known not to fit the cap: no tables are made for that (a state may be written often)
-  auto over = [&](size_t need) { return h->max_bytes && h->bytes + need > h->max_bytes; };
+  // known not to fit the cap, with room for the arrays of a written state beside them (which would
+  // push them out again): no tables are made for that (a state may be written often)
+  const size_t written = (size_t)std::max(1, h->nt) * 21 + 4;
+  auto over = [&](size_t need) { return h->max_bytes && h->bytes + need + written > h->max_bytes; };
   if (!now && over(h->seg_need)) return fail(h, SIM_ENOMEM, "device memory cap (sim_params.max_device_bytes) reached");
   std::vector<int32_t> cap;
   seg_capacities(nl, h->len.data(), h->lanes.data(), h->nt, vmin, now, cap);

@@ -74,26 +74,55 @@ def test_assignment_keeps_the_segments(G):
     assert g.launch_count() - n0 == 2 * 4
 
 
-def test_written_state_without_room_for_segments(G):
-    # finding no room for the segments costs a written state no more than laying them out does
-    sc = _grid(n=128, lanes=3, n_trips=2000)
+def _launches(g):
+    n0 = g.launch_count()
+    g.step(4)
+    return g.launch_count() - n0
+
+
+def _write_time(G, sc, cap):
+    """Seconds of a written state, and the launches of four steps after it."""
     n = sc["demand"]["n_trips"]
     st = dict(status=np.zeros(n, np.uint8), link=np.zeros(n, np.int32), lane=np.zeros(n, np.int32),
               cursor=np.zeros(n, np.int32), x=np.zeros(n, np.float32), v=np.zeros(n, np.float32))
+    g = G.Sim(_capped(sc, cap))
+    g.set_routes(sc["routes"]["offsets"], sc["routes"]["links"])
     took = []
-    for cap in (0, _least(G, sc) + (4 << 20)):
-        g = G.Sim(_capped(sc, cap))
-        g.set_routes(sc["routes"]["offsets"], sc["routes"]["links"])
-        one = []
-        for _ in range(12):
-            t = time.perf_counter()
-            g.write_state(st)
-            one.append(time.perf_counter() - t)
-        took.append(np.median(one))
-        n0 = g.launch_count()
-        g.step(4)
-        assert g.launch_count() - n0 == (2 * 4 + 1, 7 * 4)[cap > 0]
-    assert took[1] < 2.0 * took[0], took
+    for _ in range(12):
+        t = time.perf_counter()
+        g.write_state(st)
+        took.append(time.perf_counter() - t)
+    return np.median(took), _launches(g)
+
+
+def test_written_state_without_room_for_segments(G):
+    # finding no room for the segments costs a written state no more than laying them out does
+    sc = _grid(n=128, lanes=3, n_trips=2000)
+    free, launches = _write_time(G, sc, 0)
+    assert launches == 2 * 4 + 1
+    capped, launches = _write_time(G, sc, _least(G, sc) + (4 << 20))
+    assert launches == 7 * 4
+    assert capped < 2.0 * free, (capped, free)
+
+
+def test_written_state_with_just_room_for_segments(G):
+    # the segments are not made where the arrays of a written state would push them out again
+    sc = _grid(n=128, lanes=3, n_trips=20000)
+    lo = hi = _least(G, sc)
+    hi += 1 << 30
+    while hi - lo > 1024:
+        mid = (lo + hi) // 2
+        g = G.Sim(_capped(sc, mid))
+        try:
+            g.set_routes(sc["routes"]["offsets"], sc["routes"]["links"])
+            segments = _launches(g) == 2 * 4 + 1
+        except G.SimError:
+            segments = False
+        g.close()
+        lo, hi = (lo, mid) if segments else (mid, hi)
+    free, _ = _write_time(G, sc, 0)
+    capped, _ = _write_time(G, sc, hi)
+    assert capped < 2.0 * free, (capped, free)
 
 
 def test_routes_that_do_not_fit_leave_none(G):
