@@ -189,7 +189,9 @@ int sim_step(sim_handle* h, int32_t n_steps);
 
 /* Advance n_steps like sim_step, but launch every kernel directly with a CUDA event
  * after each one, and add each kernel's device time (ms, including its launch gap)
- * into kernel_ms[SIM_N_KERNELS] (host array, zeroed first).  Results are identical
+ * into kernel_ms[SIM_N_KERNELS] (host array, zeroed first).  Networks of 2,048 lanes and
+ * more that step in link segments (sim_set_exec) have two kernels: "front" holds the lane
+ * fronts, "chunk" the move phase.  Results are identical
  * to sim_step.  For profiling; slower than sim_step's graph launch. */
 int sim_step_timed(sim_handle* h, int32_t n_steps, float* kernel_ms);
 
