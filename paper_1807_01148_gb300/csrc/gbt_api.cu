@@ -258,7 +258,7 @@ int upload(sim_handle* h, T** p, const T* src, size_t n) {
 // form at any size: us per step with the reads of the state, calls of 20 steps, sorted ->
 // segments: ring of 50 vehicles (calls of 10) 23.5 -> 13.6; grids of 6 x 6 (240 lanes) 22.8 ->
 // 13.8, 10 x 10 (720) 29.2 -> 15.9, 14 x 14 (1,456) 32.6 -> 17.0, 16 x 16 (1,920) 33.5 -> 18.0;
-// and above the line 20 x 20 (3,040 lanes, 2,050 vehicles) 43.0 -> 18.5; town of 6,700
+// and above the line 20 x 20 (3,040 lanes, 2,050 vehicles) 41.3 -> 18.4; town of 6,700
 // lanes (with its share of planning) 60.1 -> 27.9; district of 42,000 lanes with outputs and
 // trucks 94 to 96 -> 86 to 90.  On networks with more groups of lanes than resident warps of the
 // move phase, in packed lists (SegDev::packed): 64 copies of a grid (321,000 lanes) 76.9 -> 62.3;
